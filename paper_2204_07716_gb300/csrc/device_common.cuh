@@ -56,24 +56,6 @@ __device__ __forceinline__ float phi<float>(int kind, int w, float beta, float z
   return (fabsf(z) <= 0.5f * float(w)) ? exp2f(-bl * z * z) : 0.f;
 }
 
-// Compact radial profile k(|u|^2) of the regression kernels (unit ball;
-// normalisation in BwDev::kscale): uniform, Epanechnikov, triangle,
-// biweight, triweight, and the Gaussian cut at Mahalanobis radius R
-// (u = z / R in the bandwidth's metric, k = exp(-R^2 |u|^2 / 2), r2 = R^2).
-template <typename T>
-__device__ __forceinline__ T compact_k(int kern, T u2, T r2) {
-  if (!(u2 <= T(1))) return T(0);
-  const T e = T(1) - u2;
-  switch (kern) {
-    case FKREG_KERNEL_UNIFORM: return T(1);
-    case FKREG_KERNEL_EPANECHNIKOV: return e;
-    case FKREG_KERNEL_TRIANGLE: return T(1) - sqrt(u2);
-    case FKREG_KERNEL_BIWEIGHT: return e * e;
-    case FKREG_KERNEL_GAUSSIAN_DIRECT: return exp(T(-0.5) * r2 * u2);
-    default: return e * e * e;
-  }
-}
-
 // Compile-time chain of the monomials of degree <= DEG in d = D variables, in
 // the graded order the plan's monomial table uses (degree by degree, index
 // multisets in lexicographic order): monomial f > 0 is monomial parent[f]
@@ -218,150 +200,6 @@ struct DirectRows {
     return true;
   }
 };
-
-// Shared memory of one warp's candidate queue in direct_warp_sums: 64
-// entries of (z[0..D), weight) in T, then 64 sample indices.
-template <typename T, int D>
-__host__ __device__ constexpr int direct_queue_bytes() {
-  return 64 * (D + 1) * int(sizeof(T)) + 64 * 4;
-}
-
-// Warp-cooperative moment sums of one evaluation point q (coordinates
-// relative to lo) over the binned samples inside its kernel support: the
-// lanes stride over the sample ranges of the support's bins (bins adjacent
-// along the last axis are one contiguous range of the sort) and test each
-// candidate; the ones inside the support are compacted into a per-warp queue
-// in shared memory (qmem, direct_queue_bytes), and each time 32 are queued
-// every lane adds one of them to all fields in registers, so that the
-// monomial and strength work runs on full warps.  The fields are reduced
-// across the warp at the end: field f is returned to lane f mod 32 (out0 for
-// f < 32, out1 above): [0, NS) the s-fields, NS + r NT + k the t-fields of
-// strength str_first + r.  NS and NT are the monomial counts of degrees 2*ORD
-// and ORD; FMAX >= NS + nstr NT bounds the fields.  Sums are in the plan
-// precision T.
-template <typename T, int D, int ORD, int FMAX>
-__device__ __forceinline__ void direct_warp_sums(const GeoDev& g, const BwDev& B, int64_t n,
-                                                 const T* __restrict__ xs,
-                                                 const T* __restrict__ str, int str_first,
-                                                 int nstr, const uint32_t* __restrict__ bin_start,
-                                                 const double* q, int lane, unsigned char* qmem,
-                                                 T& out0, T& out1) {
-  constexpr int NS = mono_count(D, 2 * ORD), NT = mono_count(D, ORD);
-  constexpr int QMAX = (FMAX - NS) / NT;
-  static_assert(QMAX >= 1 && FMAX <= 64, "field bucket");
-  T* qv = reinterpret_cast<T*>(qmem);                                   // [D + 1][64]
-  uint32_t* qi = reinterpret_cast<uint32_t*>(qmem + 64 * (D + 1) * sizeof(T));  // [64]
-  DirectRows<D> rows;
-#pragma unroll
-  for (int j = 0; j < D; ++j) rows.mn[j] = rows.mx[j] = float(q[j]);
-  rows.box(g, B);
-  T qt[D], hi[D][D];
-#pragma unroll
-  for (int a = 0; a < D; ++a) {
-    qt[a] = T(q[a]);
-#pragma unroll
-    for (int c = 0; c < D; ++c) hi[a][c] = T(B.Hinv[a * 3 + c]);
-  }
-  const T ks = T(B.kscale), kr2 = T(B.kr2);
-  const int kern = g.kern;
-  T acc[FMAX];
-#pragma unroll
-  for (int f = 0; f < FMAX; ++f) acc[f] = T(0);
-  // one queued candidate per lane (lane < cnt) into every field
-  auto consume = [&](int cnt) {
-    if (lane < cnt) {
-      T z[D];
-#pragma unroll
-      for (int j = 0; j < D; ++j) z[j] = qv[j * 64 + lane];
-      const T wgt = qv[D * 64 + lane];
-      const int64_t i = qi[lane];
-      T mo[NS];
-      mono_build<T, D, 2 * ORD>(mo, z);
-#pragma unroll
-      for (int f = 0; f < NS; ++f) acc[f] += wgt * mo[f];
-#pragma unroll
-      for (int r = 0; r < QMAX; ++r)
-        if (r < nstr) {
-          const T cw = wgt * str[int64_t(str_first + r) * n + i];
-#pragma unroll
-          for (int k = 0; k < NT; ++k) acc[NS + r * NT + k] += cw * mo[k];
-        }
-    }
-  };
-  int qn = 0;  // queued candidates (warp-uniform)
-  const unsigned below = (1u << lane) - 1u;
-  const int o0 = rows.rows0(), o1 = rows.rows1();
-  for (int r0 = 0; r0 < o0; ++r0)
-    for (int r1 = 0; r1 < o1; ++r1) {
-      int64_t first, last;  // bins [first, last] are adjacent in sorted order
-      if (!rows.row(g, r0, r1, first, last)) continue;
-      if (!in_range(g.errw, kSiteDirectBins, first, last + 1) ||
-          !in_range(g.errw, kSiteDirectBins, last, g.nbins[0] * g.nbins[1] * g.nbins[2]))
-        continue;
-      const uint32_t i1 = bin_start[last + 1];
-      for (uint32_t base = bin_start[first]; base < i1; base += 32) {
-        const uint32_t i = base + uint32_t(lane);
-        T z[D];
-        bool in = false;
-        T wgt = T(0);
-        if (i < i1) {
-#pragma unroll
-          for (int j = 0; j < D; ++j) z[j] = xs[int64_t(j) * n + i] - qt[j];
-          T u2 = T(0);
-#pragma unroll
-          for (int a = 0; a < D; ++a) {
-            T ra = T(0);
-#pragma unroll
-            for (int c = 0; c < D; ++c) ra += hi[a][c] * z[c];
-            u2 += z[a] * ra;
-          }
-          in = u2 <= T(1);
-          if (in) wgt = ks * compact_k<T>(kern, u2, kr2);
-        }
-        const unsigned m = __ballot_sync(0xffffffffu, in);
-        if (in) {
-          const int slot = qn + __popc(m & below);
-#pragma unroll
-          for (int j = 0; j < D; ++j) qv[j * 64 + slot] = z[j];
-          qv[D * 64 + slot] = wgt;
-          qi[slot] = i;
-        }
-        qn += __popc(m);
-        if (qn >= 32) {
-          __syncwarp();
-          consume(32);
-          __syncwarp();
-          if (lane < qn - 32) {  // move the overflow to the front of the queue
-#pragma unroll
-            for (int j = 0; j <= D; ++j) qv[j * 64 + lane] = qv[j * 64 + 32 + lane];
-            qi[lane] = qi[32 + lane];
-          }
-          qn -= 32;
-          __syncwarp();
-        }
-      }
-    }
-  __syncwarp();
-  consume(qn);
-  __syncwarp();
-  out0 = T(0);
-  out1 = T(0);
-  const int nf = NS + nstr * NT;
-#pragma unroll
-  for (int f = 0; f < FMAX; ++f) {
-    if (f < nf) {
-      T v = acc[f];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == (f & 31)) {
-        if (f < 32)
-          out0 = v;
-        else
-          out1 = v;
-      }
-    }
-  }
-}
 
 template <typename T>
 __device__ __forceinline__ T sel3(int ax, T a, T b, T c) {

@@ -50,6 +50,10 @@ struct GeoDev {
 // Bits of the plan's device error word.
 constexpr int kErrOutside = 1;  // a sample outside the grid box or not finite
 constexpr int kErrTimeout = 2;  // a bounded device-side wait gave up
+// Word errw[kStrFlag] of the direct path: the number (fkreg_plan_s::str_pass) of
+// the last strengths pass in which a value was not finite.
+constexpr int kStrFlag = 16;
+constexpr int kTaskWord = 17;  // next group of targets of the direct at-sample pass
 constexpr int kErrBounds = 4;   // a bounds check of the checked build failed (access skipped)
 
 // Sort keys are (bin << kbits) | local, local = serpentine index of the
@@ -145,6 +149,7 @@ struct fkreg_plan_s {
   int device = -1;
 
   // profiling: own kernel launches, per-stage events
+  int str_pass = 0;             // direct path: strengths passes so far
   int64_t launches = 0;
   bool timing = false;
   struct Pending {

@@ -605,12 +605,24 @@ __global__ void kernel_values_kernel(int kind, int w, T beta, int64_t n, const T
   if (i < n) out[i] = phi<T>(kind, w, beta, z[i]);
 }
 
+// Stores a strength; the direct path (word != null) notes one that is not
+// finite under this pass's number.
+struct StrFlag {
+  int* word;
+  int pass;
+  template <typename T>
+  __device__ __forceinline__ void put(T& to, T v) const {
+    to = v;
+    if (word && !isfinite(v)) *word = pass;
+  }
+};
+
 template <typename T>
 __global__ void gather_strengths_kernel(int64_t n, const uint32_t* __restrict__ perm,
                                         const T* __restrict__ y, int n_rhs, int y_complex,
                                         int with_density, int n_probes, uint64_t seed,
                                         const T* __restrict__ probes, T* __restrict__ str,
-                                        int first) {
+                                        int first, StrFlag flag) {
   const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (s >= n) return;
   const uint32_t i = perm[s];
@@ -618,14 +630,15 @@ __global__ void gather_strengths_kernel(int64_t n, const uint32_t* __restrict__ 
   if (with_density) str[int64_t(k++) * n + s] = T(1);
   for (int r = 0; r < n_rhs; ++r) {
     if (y_complex) {
-      str[int64_t(k++) * n + s] = y[(int64_t(r) * n + i) * 2 + 0];
-      str[int64_t(k++) * n + s] = y[(int64_t(r) * n + i) * 2 + 1];
+      flag.put(str[int64_t(k++) * n + s], y[(int64_t(r) * n + i) * 2 + 0]);
+      flag.put(str[int64_t(k++) * n + s], y[(int64_t(r) * n + i) * 2 + 1]);
     } else {
-      str[int64_t(k++) * n + s] = y[int64_t(r) * n + i];
+      flag.put(str[int64_t(k++) * n + s], y[int64_t(r) * n + i]);
     }
   }
   if (probes) {
-    for (int p = 0; p < n_probes; ++p) str[int64_t(k++) * n + s] = probes[int64_t(p) * n + i];
+    for (int p = 0; p < n_probes; ++p)
+      flag.put(str[int64_t(k++) * n + s], probes[int64_t(p) * n + i]);
   } else {
     for (int p = 0; p < n_probes; p += 2) {
       T z0, z1;
@@ -641,7 +654,7 @@ template <typename T>
 __global__ void residual_strengths_kernel(int64_t n, const uint32_t* __restrict__ perm,
                                           const T* __restrict__ y, const T* __restrict__ mh,
                                           int n_rhs, int y_complex, int b, T* __restrict__ str,
-                                          int first) {
+                                          int first, StrFlag flag) {
   const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (s >= n) return;
   const uint32_t i = perm[s];
@@ -656,7 +669,7 @@ __global__ void residual_strengths_kernel(int64_t n, const uint32_t* __restrict_
       const T dr = y[int64_t(r) * n + i] - mh[(int64_t(b) * n_rhs + r) * n + i];
       v = dr * dr;
     }
-    str[int64_t(first + r) * n + s] = v;
+    flag.put(str[int64_t(first + r) * n + s], v);
   }
 }
 
@@ -665,18 +678,24 @@ __global__ void residual_strengths_kernel(int64_t n, const uint32_t* __restrict_
 template <typename T>
 __global__ void logres_strengths_kernel(int64_t n, const uint32_t* __restrict__ perm,
                                         const T* __restrict__ y, const T* __restrict__ mh,
-                                        int n_rhs, int b, T* __restrict__ str, int first) {
+                                        int n_rhs, int b, T* __restrict__ str, int first,
+                                        StrFlag flag) {
   const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (s >= n) return;
   const uint32_t i = perm[s];
   const T inv_n = T(1) / T(n);
   for (int r = 0; r < n_rhs; ++r) {
     const T dr = y[int64_t(r) * n + i] - mh[(int64_t(b) * n_rhs + r) * n + i];
-    str[int64_t(first + r) * n + s] = log(dr * dr + inv_n);
+    flag.put(str[int64_t(first + r) * n + s], log(dr * dr + inv_n));
   }
 }
 
 }  // namespace
+
+static StrFlag next_pass(fkreg_plan_s* P) {
+  if (!P->direct) return StrFlag{nullptr, 0};
+  return StrFlag{wsp<int>(P, P->r_err) + kStrFlag, ++P->str_pass};
+}
 
 const uint32_t* perm_ptr(fkreg_plan_s* P) {
   return P->perm_in_vals1 ? wsp<uint32_t>(P, P->r_vals1) : wsp<uint32_t>(P, P->r_vals0);
@@ -697,14 +716,15 @@ cudaError_t run_gather_strengths(fkreg_plan_s* P, const void* y, int first_str, 
   if (P->n == 0) return cudaSuccess;
   const unsigned blocks = unsigned((P->n + 255) / 256);
   const uint32_t* perm = perm_ptr(P);
+  const StrFlag flag = next_pass(P);
   if (P->prec == FKREG_F32)
     gather_strengths_kernel<float><<<blocks, 256, 0, st>>>(
         P->n, perm, static_cast<const float*>(y), P->nrhs, P->o.y_complex, with_density, n_probes,
-        seed, static_cast<const float*>(probes), wsp<float>(P, P->r_str), first_str);
+        seed, static_cast<const float*>(probes), wsp<float>(P, P->r_str), first_str, flag);
   else
     gather_strengths_kernel<double><<<blocks, 256, 0, st>>>(
         P->n, perm, static_cast<const double*>(y), P->nrhs, P->o.y_complex, with_density, n_probes,
-        seed, static_cast<const double*>(probes), wsp<double>(P, P->r_str), first_str);
+        seed, static_cast<const double*>(probes), wsp<double>(P, P->r_str), first_str, flag);
   P->launches += 1;
   return cudaGetLastError();
 }
@@ -714,14 +734,15 @@ cudaError_t run_residual_strengths(fkreg_plan_s* P, const void* y, const void* m
   if (P->n == 0) return cudaSuccess;
   const unsigned blocks = unsigned((P->n + 255) / 256);
   const uint32_t* perm = perm_ptr(P);
+  const StrFlag flag = next_pass(P);
   if (P->prec == FKREG_F32)
     residual_strengths_kernel<float><<<blocks, 256, 0, st>>>(
         P->n, perm, static_cast<const float*>(y), static_cast<const float*>(mhat_at_x), P->nrhs,
-        P->o.y_complex, b, wsp<float>(P, P->r_str), first_str);
+        P->o.y_complex, b, wsp<float>(P, P->r_str), first_str, flag);
   else
     residual_strengths_kernel<double><<<blocks, 256, 0, st>>>(
         P->n, perm, static_cast<const double*>(y), static_cast<const double*>(mhat_at_x), P->nrhs,
-        P->o.y_complex, b, wsp<double>(P, P->r_str), first_str);
+        P->o.y_complex, b, wsp<double>(P, P->r_str), first_str, flag);
   P->launches += 1;
   return cudaGetLastError();
 }
@@ -735,14 +756,15 @@ cudaError_t run_logres_strengths(fkreg_plan_s* P, const void* y, const void* mha
   if (P->n == 0) return cudaSuccess;
   const unsigned blocks = unsigned((P->n + 255) / 256);
   const uint32_t* perm = perm_ptr(P);
+  const StrFlag flag = next_pass(P);
   if (P->prec == FKREG_F32)
     logres_strengths_kernel<float><<<blocks, 256, 0, st>>>(
         P->n, perm, static_cast<const float*>(y), static_cast<const float*>(mhat_at_x), P->nrhs,
-        b, wsp<float>(P, P->r_str), first_str);
+        b, wsp<float>(P, P->r_str), first_str, flag);
   else
     logres_strengths_kernel<double><<<blocks, 256, 0, st>>>(
         P->n, perm, static_cast<const double*>(y), static_cast<const double*>(mhat_at_x), P->nrhs,
-        b, wsp<double>(P, P->r_str), first_str);
+        b, wsp<double>(P, P->r_str), first_str, flag);
   P->launches += 1;
   return cudaGetLastError();
 }
