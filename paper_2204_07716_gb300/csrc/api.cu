@@ -267,7 +267,6 @@ fkreg_status fkreg_plan_create(const fkreg_opts* opts, int64_t max_n, fkreg_plan
   int64_t nb = 1;
   for (int a = 0; a < d; ++a) nb *= P->g.nbins[a];
   P->nbins_total = nb;
-  P->nsub_max = nb + (max_n + fk::kSubMax - 1) / fk::kSubMax;
   // device and its SM count (persistent grids are sized from it)
   if (cudaGetDevice(&P->device) != cudaSuccess ||
       cudaDeviceGetAttribute(&P->sm_count, cudaDevAttrMultiProcessorCount, P->device) !=
@@ -277,6 +276,7 @@ fkreg_status fkreg_plan_create(const fkreg_opts* opts, int64_t max_n, fkreg_plan
     return set_global_error(FKREG_ERR_CUDA, "no CUDA device");
   }
   P->nblk_interp = int64_t(P->sm_count) * 8;
+  P->nsub_max = nb + (max_n + fk::kSubMax - 1) / fk::kSubMax;
   // tile + halo must fit shared memory for one strength
   {
     size_t cells = 1;
@@ -328,7 +328,7 @@ fkreg_status fkreg_plan_create(const fkreg_opts* opts, int64_t max_n, fkreg_plan
   }
   L.take(P->r_t2spec, std::max<int64_t>(256, fft_scale * 2 * T * int64_t(t2_fields) * t2_half));
   L.take(P->r_t2field,
-         std::max<int64_t>(256, fft_scale * T * int64_t(fk::t2_record_stride(t2_fields)) * t2_cells));
+         std::max<int64_t>(256, fft_scale * T * int64_t(fk::t2_record_stride(t2_fields, T)) * t2_cells));
   L.take(P->r_part, sizeof(double) * size_t(P->nblk_interp + 1) * P->nbw * P->nacc);
   L.take(P->r_smax, 8 * size_t(P->nbw));
   if (P->backward) {

@@ -56,6 +56,14 @@ __device__ __forceinline__ float phi<float>(int kind, int w, float beta, float z
   return (fabsf(z) <= 0.5f * float(w)) ? exp2f(-bl * z * z) : 0.f;
 }
 
+// All W kernel values phi(off + t), t = 0 .. W-1, of one axis (off is the first
+// cell's offset, in [-w/2, -w/2 + 1)).
+template <int W, typename T>
+__device__ __forceinline__ void phi_row(int skind, T beta, T off, T (&v)[W]) {
+#pragma unroll
+  for (int t = 0; t < W; ++t) v[t] = phi<T>(skind, W, beta, off + T(t));
+}
+
 // Compile-time chain of the monomials of degree <= DEG in d = D variables, in
 // the graded order the plan's monomial table uses (degree by degree, index
 // multisets in lexicographic order): monomial f > 0 is monomial parent[f]
@@ -216,43 +224,92 @@ __device__ __forceinline__ T warp_sum_t(T v) {
   return v;
 }
 
-// Solve S a = e_1 (p x p, FP64, partial pivoting). Returns false if singular.
-__device__ __forceinline__ bool solve_e1(int p, double S[kMaxP][kMaxP], double a[kMaxP]) {
-  double r[kMaxP];
-  for (int i = 0; i < p; ++i) r[i] = (i == 0) ? 1.0 : 0.0;
-  for (int c = 0; c < p; ++c) {
-    int piv = c;
-    for (int i = c + 1; i < p; ++i)
-      if (fabs(S[i][c]) > fabs(S[piv][c])) piv = i;
-    if (!(fabs(S[piv][c]) > 0.0)) return false;
-    if (piv != c) {
-      for (int j = 0; j < p; ++j) {
-        double t = S[c][j];
-        S[c][j] = S[piv][j];
-        S[piv][j] = t;
-      }
-      double t = r[c];
-      r[c] = r[piv];
-      r[piv] = t;
-    }
-    for (int i = c + 1; i < p; ++i) {
-      const double f = S[i][c] / S[c][c];
-      for (int j = c; j < p; ++j) S[i][j] -= f * S[c][j];
-      r[i] -= f * r[c];
-    }
-  }
-  for (int i = p - 1; i >= 0; --i) {
-    double v = r[i];
-    for (int j = i + 1; j < p; ++j) v -= S[i][j] * a[j];
-    a[i] = v / S[i][i];
-  }
-  return isfinite(a[0]);
-}
-
 __device__ __forceinline__ int mono_index(const MonoTab& m, int nm, int e0, int e1, int e2) {
   for (int k = 0; k < nm; ++k)
     if (m.e[k][0] == e0 && m.e[k][1] == e1 && m.e[k][2] == e2) return k;
   return 0;
+}
+
+// The normal matrix of a D-variate system of order ORD at compile time: s[i][j]
+// is the s-field of the product of the t-monomials i and j (the graded order
+// of make_mono_chain), ax[i] the axes of t-monomial i (-1 past its degree).
+template <int D, int ORD>
+struct LprTab {
+  int s[mono_count(D, ORD)][mono_count(D, ORD)];
+  int ax[mono_count(D, ORD)][2];
+};
+template <int D, int ORD>
+__host__ __device__ constexpr LprTab<D, ORD> make_lpr_tab() {
+  constexpr int P = mono_count(D, ORD);
+  const MonoChain c = make_mono_chain(D, 2 * ORD);
+  int e[kMaxMono][3] = {};
+  for (int f = 1; f < c.n; ++f) {
+    for (int j = 0; j < 3; ++j) e[f][j] = e[c.parent[f]][j];
+    e[f][c.axis[f]] += 1;
+  }
+  LprTab<D, ORD> t{};
+  for (int i = 0; i < P; ++i) {
+    int n = 0;
+    t.ax[i][0] = t.ax[i][1] = -1;
+    for (int j = 0; j < 3; ++j)
+      for (int r = 0; r < e[i][j]; ++r) t.ax[i][n++] = j;
+    for (int j = 0; j < P; ++j)
+      for (int f = 0; f < c.n; ++f)
+        if (e[f][0] == e[i][0] + e[j][0] && e[f][1] == e[i][1] + e[j][1] &&
+            e[f][2] == e[i][2] + e[j][2])
+          t.s[i][j] = f;
+  }
+  return t;
+}
+
+// S a = e_1 (P x P, FP64) by elimination with partial pivoting, every index
+// known at compile time (the columns are unrolled by recursion) so that S stays
+// in registers: the largest entry of a column is brought up by conditional
+// swaps (integer selects, next to nothing on the 2-lane FP64 pipe of an SM)
+// and each pivot costs one division.  With S in local memory and runtime
+// indices the 6 x 6 systems of 300,007 samples took most of a 0.77 ms kernel.
+// solve_e1 returns false if S is singular.
+template <int P, int C>
+__device__ __forceinline__ bool eliminate(double (&S)[P][P], double (&r)[P], double* a) {
+  if constexpr (C == P) {
+    return true;
+  } else {
+#pragma unroll
+    for (int i = C + 1; i < P; ++i) {
+      const bool up = fabs(S[i][C]) > fabs(S[C][C]);
+#pragma unroll
+      for (int j = C; j < P; ++j) {
+        const double t = S[C][j];
+        S[C][j] = up ? S[i][j] : t;
+        S[i][j] = up ? t : S[i][j];
+      }
+      const double t = r[C];
+      r[C] = up ? r[i] : t;
+      r[i] = up ? t : r[i];
+    }
+    const bool ok = fabs(S[C][C]) > 0.0;
+    const double inv = 1.0 / S[C][C];
+#pragma unroll
+    for (int i = C + 1; i < P; ++i) {
+      const double f = S[i][C] * inv;
+#pragma unroll
+      for (int j = C + 1; j < P; ++j) S[i][j] -= f * S[C][j];
+      r[i] -= f * r[C];
+    }
+    const bool rest = eliminate<P, C + 1>(S, r, a);
+    double v = r[C];
+#pragma unroll
+    for (int j = C + 1; j < P; ++j) v -= S[C][j] * a[j];
+    a[C] = v * inv;
+    return ok && rest;
+  }
+}
+template <int P>
+__device__ __forceinline__ bool solve_e1(double (&S)[P][P], double* a) {
+  double r[P];
+#pragma unroll
+  for (int i = 0; i < P; ++i) r[i] = (i == 0) ? 1.0 : 0.0;
+  return eliminate<P, 0>(S, r, a) && isfinite(a[0]);
 }
 
 // sigma^g for the t-field monomial a
@@ -263,37 +320,30 @@ __device__ __forceinline__ double tscale(const MonoTab& mono, int a, const doubl
   return sc;
 }
 
-// Scaled normal matrix S~_ab = s_(a+b) / sigma^(a+b) from the s-fields, and
-// a = S~^-1 e_1 (the intercept is unchanged by the scaling), by elimination.
-__device__ __forceinline__ bool lpr_weights(const MonoTab& mono, int p, const double* s,
-                                            const double* sigma, double a[kMaxP]) {
-  double S[kMaxP][kMaxP];
-  for (int i = 0; i < p; ++i)
-    for (int j = 0; j < p; ++j) {
-      const int e0 = mono.e[i][0] + mono.e[j][0];
-      const int e1 = mono.e[i][1] + mono.e[j][1];
-      const int e2 = mono.e[i][2] + mono.e[j][2];
-      const int k = mono_index(mono, mono.n, e0, e1, e2);
-      double sc = 1.0;
-      for (int r = 0; r < e0; ++r) sc *= sigma[0];
-      for (int r = 0; r < e1; ++r) sc *= sigma[1];
-      for (int r = 0; r < e2; ++r) sc *= sigma[2];
-      S[i][j] = s[k] / sc;
-    }
-  return solve_e1(p, S, a);
+// its[i] = 1 / sigma^g of t-monomial i from isg = 1 / sigma.
+template <int D, int ORD>
+__device__ __forceinline__ void lpr_iscale(const double* isg, double* its) {
+  constexpr auto tab = make_lpr_tab<D, ORD>();
+#pragma unroll
+  for (int i = 0; i < mono_count(D, ORD); ++i) {
+    double sc = 1.0;
+#pragma unroll
+    for (int w = 0; w < 2; ++w)
+      if (tab.ax[i][w] >= 0) sc *= isg[tab.ax[i][w]];
+    its[i] = sc;
+  }
 }
 
-// Same result with closed forms for Nadaraya-Watson and local linear in 1-D
-// and 2-D (one division); isg = 1 / sigma.  Other systems (local linear in
-// 3-D, local quadratic) go through elimination.
-__device__ __forceinline__ bool lpr_weights_fast(const MonoTab& mono, int p, const double* s,
-                                                 const double* sigma, const double* isg,
-                                                 double a[kMaxP]) {
-  if (p == 1) {
+// a = S~^-1 e_1 of the scaled normal matrix S~_ab = s_(a+b) / sigma^(a+b)
+// (the intercept is unchanged by the scaling), isg = 1 / sigma: closed forms
+// for Nadaraya-Watson and local linear in 1-D and 2-D (one division),
+// elimination for local linear in 3-D and local quadratic.
+template <int D, int ORD>
+__device__ __forceinline__ bool lpr_weights(const double* s, const double* isg, double* a) {
+  if constexpr (ORD == 0) {
     a[0] = 1.0 / s[0];
     return s[0] > 0.0;
-  }
-  if (p == 2 && mono.n == 3) {  // 1-D local linear
+  } else if constexpr (D == 1 && ORD == 1) {
     const double s01 = s[1] * isg[0], s11 = s[2] * (isg[0] * isg[0]);
     const double det = s[0] * s11 - s01 * s01;
     if (!(det > 0.0)) return false;
@@ -301,8 +351,7 @@ __device__ __forceinline__ bool lpr_weights_fast(const MonoTab& mono, int p, con
     a[0] = s11 * inv;
     a[1] = -s01 * inv;
     return isfinite(a[0]);
-  }
-  if (p == 3 && mono.n == 6) {  // 2-D local linear, s-fields 1, z1, z2, z1z1, z1z2, z2z2
+  } else if constexpr (D == 2 && ORD == 1) {
     const double h0 = isg[0], h1 = isg[1];
     const double s00 = s[0], s01 = s[1] * h0, s02 = s[2] * h1;
     const double s11 = s[3] * (h0 * h0), s12 = s[4] * (h0 * h1), s22 = s[5] * (h1 * h1);
@@ -316,8 +365,36 @@ __device__ __forceinline__ bool lpr_weights_fast(const MonoTab& mono, int p, con
     a[1] = c1 * inv;
     a[2] = c2 * inv;
     return isfinite(a[0]);
+  } else {
+    constexpr int P = mono_count(D, ORD);
+    constexpr auto tab = make_lpr_tab<D, ORD>();
+    double S[P][P], its[P];
+    lpr_iscale<D, ORD>(isg, its);
+#pragma unroll
+    for (int i = 0; i < P; ++i)
+#pragma unroll
+      for (int j = i; j < P; ++j) S[i][j] = S[j][i] = s[tab.s[i][j]] * (its[i] * its[j]);
+    return solve_e1<P>(S, a);
   }
-  return lpr_weights(mono, p, s, sigma, a);
+}
+
+// The same for an order known at run time (3-D plans have orders 0 and 1).
+// Eliminations are a call: inlined, their registers spilled the gathers of the
+// 512-thread kernels that hold this (3-D local linear 3.8 -> 6.2 ms).
+template <int D, int ORD>
+__device__ __noinline__ bool lpr_weights_call(const double* s, const double* isg, double* a) {
+  return lpr_weights<D, ORD>(s, isg, a);
+}
+template <int D>
+__device__ __forceinline__ bool lpr_weights_order(int order, const double* s, const double* isg,
+                                                  double* a) {
+  if (order == 0) return lpr_weights<D, 0>(s, isg, a);
+  if constexpr (D < 3) {
+    if (order == 2) return lpr_weights_call<D, 2>(s, isg, a);
+    return lpr_weights<D, 1>(s, isg, a);
+  } else {
+    return lpr_weights_call<D, 1>(s, isg, a);
+  }
 }
 
 // ---- compensated FP32 arithmetic for the at-sample solves ------------------

@@ -459,8 +459,8 @@ direct_sums_kernel(GeoDev g, MonoTab mono, DsArgs a, const BwDev* __restrict__ b
 #pragma unroll
         for (int k = 0; k < kMaxP; ++k)
           tsc[k] = (k < c.p) ? T(1.0 / tscale(mono, k, B.sigma)) : T(0);
-        const double isg[3] = {1.0 / B.sigma[0], 1.0 / B.sigma[1], 1.0 / B.sigma[2]};
-        finish_pass<T>(c, mono, B, my, 0, 0, c.nq, lane, valid, n, str + n + s, n,
+        const double isg[3] = {B.isigma[0], B.isigma[1], B.isigma[2]};
+        finish_pass<T, D, ORD>(c, mono, B, my, 0, 0, c.nq, lane, valid, n, str + n + s, n,
                                valid ? perm[s] : 0u, mhat_at_x, tsc, af, red, T(B.k0), isg);
       }
       // the groups of a dense region cost tens of times those of a sparse one: the

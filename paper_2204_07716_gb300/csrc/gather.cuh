@@ -1,5 +1,5 @@
 // Per-sample window geometry and the warp-cooperative gather of interleaved
-// fields, shared by the interpolation and backward kernels.
+// fields, for the interpolation kernel of runtime widths.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -50,8 +50,8 @@ __device__ __forceinline__ SampleWin<T, D> sample_window(const GeoDev& g, int w,
 }
 
 // Gather fields [f_first, f_first + fcount) of one sample from the global
-// field grid (periodic wrap).  Lanes cover the fields.
-template <typename T, int D, int W, int NCH>
+// field grid (periodic wrap), any window width.  Lanes cover the fields.
+template <typename T, int D, int NCH>
 __device__ __forceinline__ void gather_global(const T* __restrict__ fld, int64_t rec, int f_first,
                                               int fcount, int lane, const SampleWin<T, D>& sw,
                                               int w, int nf0, int nf1, int nf2, T* cellw,
@@ -59,100 +59,42 @@ __device__ __forceinline__ void gather_global(const T* __restrict__ fld, int64_t
 #pragma unroll
   for (int ch = 0; ch < NCH; ++ch) acc[ch] = T(0);
   const T* fb = fld + f_first + lane;
-  if constexpr (W > 0) {
-    T wa[D][W];
-#pragma unroll
-    for (int d = 0; d < D; ++d)
-#pragma unroll
-      for (int t = 0; t < W; ++t) {
-        const int l = d * W + t;
-        wa[d][t] = l < 32 ? __shfl_sync(0xffffffffu, sw.wl0, l) : __shfl_sync(0xffffffffu, sw.wl1, l - 32);
-      }
-    const int ilast = D == 1 ? sw.i0 : (D == 2 ? sw.i1 : sw.i2);
-    const int nlast = D == 1 ? nf0 : (D == 2 ? nf1 : nf2);
-    int64_t clf[W];
-#pragma unroll
-    for (int t = 0; t < W; ++t) clf[t] = wrap_idx(ilast + t, nlast) * rec;
-    if (D == 1) {
-#pragma unroll
-      for (int t0 = 0; t0 < W; ++t0) {
-        const T* q = fb + clf[t0];
-        const T v = wa[0][t0];
-#pragma unroll
-        for (int ch = 0; ch < NCH; ++ch)
-          if (lane + ch * 32 < fcount) acc[ch] += __ldg(q + ch * 32) * v;
-      }
-    } else if (D == 2) {
-#pragma unroll
-      for (int t0 = 0; t0 < W; ++t0) {
-        const T* rowp = fb + wrap_idx(sw.i0 + t0, nf0) * nf1 * rec;
-        const T w0 = wa[0][t0];
-#pragma unroll
-        for (int t1 = 0; t1 < W; ++t1) {
-          const T* q = rowp + clf[t1];
-          const T v = w0 * wa[D - 1][t1];
-#pragma unroll
-          for (int ch = 0; ch < NCH; ++ch)
-            if (lane + ch * 32 < fcount) acc[ch] += __ldg(q + ch * 32) * v;
-        }
-      }
-    } else {
-#pragma unroll 1
-      for (int t0 = 0; t0 < W; ++t0) {
-        const int64_t r0 = wrap_idx(sw.i0 + t0, nf0) * nf1;
-#pragma unroll
-        for (int t1 = 0; t1 < W; ++t1) {
-          const T* rowp = fb + (r0 + wrap_idx(sw.i1 + t1, nf1)) * nf2 * rec;
-          const T w01 = wa[0][t0] * wa[1 % D][t1];
-#pragma unroll
-          for (int t2 = 0; t2 < W; ++t2) {
-            const T* q = rowp + clf[t2];
-            const T v = w01 * wa[D - 1][t2];
-#pragma unroll
-            for (int ch = 0; ch < NCH; ++ch)
-              if (lane + ch * 32 < fcount) acc[ch] += __ldg(q + ch * 32) * v;
-          }
-        }
-      }
+  // tensor-product cell weights through shared memory
+  int ncw = 1;
+  for (int j = 0; j < D; ++j) ncw *= w;
+  for (int c0 = 0; c0 < ncw; c0 += 32) {
+    const int c = c0 + lane;
+    int rem = c < ncw ? c : 0;
+    T v = T(1);
+    for (int d = D - 1; d >= 0; --d) {
+      const int t = rem % w;
+      rem /= w;
+      const int l = d * w + t;
+      const T a0 = __shfl_sync(0xffffffffu, sw.wl0, l & 31);
+      const T a1 = __shfl_sync(0xffffffffu, sw.wl1, l & 31);
+      v *= (l < 32) ? a0 : a1;
     }
-  } else {
-    // runtime width: tensor-product cell weights through shared memory
-    int ncw = 1;
-    for (int j = 0; j < D; ++j) ncw *= w;
-    for (int c0 = 0; c0 < ncw; c0 += 32) {
-      const int c = c0 + lane;
-      int rem = c < ncw ? c : 0;
-      T v = T(1);
-      for (int d = D - 1; d >= 0; --d) {
-        const int t = rem % w;
-        rem /= w;
-        const int l = d * w + t;
-        const T a0 = __shfl_sync(0xffffffffu, sw.wl0, l & 31);
-        const T a1 = __shfl_sync(0xffffffffu, sw.wl1, l & 31);
-        v *= (l < 32) ? a0 : a1;
-      }
-      if (c < ncw) cellw[c] = v;
-    }
-    __syncwarp();
-    for (int c = 0; c < ncw; ++c) {
-      int rem = c;
-      int64_t cell = 0, mult = 1;
-      for (int d = D - 1; d >= 0; --d) {
-        const int t = rem % w;
-        rem /= w;
-        const int id = d == 0 ? sw.i0 : (d == 1 ? sw.i1 : sw.i2);
-        const int nfd = d == 0 ? nf0 : (d == 1 ? nf1 : nf2);
-        cell += wrap_idx(id + t, nfd) * mult;
-        mult *= nfd;
-      }
-      const T* q = fb + cell * rec;
-      const T v = cellw[c];
-#pragma unroll
-      for (int ch = 0; ch < NCH; ++ch)
-        if (lane + ch * 32 < fcount) acc[ch] += q[ch * 32] * v;
-    }
-    __syncwarp();
+    if (c < ncw) cellw[c] = v;
   }
+  __syncwarp();
+  for (int c = 0; c < ncw; ++c) {
+    int rem = c;
+    int64_t cell = 0, mult = 1;
+    for (int d = D - 1; d >= 0; --d) {
+      const int t = rem % w;
+      rem /= w;
+      const int id = d == 0 ? sw.i0 : (d == 1 ? sw.i1 : sw.i2);
+      const int nfd = d == 0 ? nf0 : (d == 1 ? nf1 : nf2);
+      cell += wrap_idx(id + t, nfd) * mult;
+      mult *= nfd;
+    }
+    const T* q = fb + cell * rec;
+    const T v = cellw[c];
+#pragma unroll
+    for (int ch = 0; ch < NCH; ++ch)
+      if (lane + ch * 32 < fcount) acc[ch] += q[ch * 32] * v;
+  }
+  __syncwarp();
 }
 
 }  // namespace fk

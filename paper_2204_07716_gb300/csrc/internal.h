@@ -76,6 +76,7 @@ inline int key_local_bits(int d, const int64_t* tile, const int64_t* nbins) {
 struct BwDev {
   double H[9];
   double sigma[3];     // sqrt(H_jj)
+  double isigma[3];    // 1 / sigma
   double k0;           // K_H(0)
   int64_t K[3];        // modes this bandwidth needs
   int64_t nf[3];       // type-2 fine grid for this bandwidth
@@ -223,6 +224,14 @@ cudaError_t run_gather_fields(fkreg_plan_s* P, int b, int F, void* V, cudaStream
 cudaError_t run_interp_direct(fkreg_plan_s* P, int b, int n_rhs_real, int n_probes,
                               void* mhat_at_x, cudaStream_t st, int nacc, int F2, void* vout,
                               bool* launched);
+// Lane-per-sample kernels of interp_lane.cuh (compile-time widths, every
+// dimension and order), launched only when they apply (*launched).
+cudaError_t run_interp_lane_f32(fkreg_plan_s* P, int b, int n_rhs_real, int n_probes,
+                                void* mhat_at_x, cudaStream_t st, int nacc, int F2, void* vout,
+                                bool* launched);
+cudaError_t run_interp_lane_f64(fkreg_plan_s* P, int b, int n_rhs_real, int n_probes,
+                                void* mhat_at_x, cudaStream_t st, int nacc, int F2, void* vout,
+                                bool* launched);
 // Lane-per-sample kernel over the global field grid (FP32, width 7, 3-D
 // Nadaraya-Watson or gather-only, F2 <= 64), launched only when it applies.
 cudaError_t run_interp_global_lane(fkreg_plan_s* P, int b, int n_rhs_real, int n_probes,
@@ -258,9 +267,9 @@ cudaError_t run_kappa_sigma2(fkreg_plan_s* P, int b, const void* y, const void* 
                              cudaStream_t s);
 
 const uint32_t* perm_ptr(fkreg_plan_s* P);
-int t2_record_stride(int F2);
+int t2_record_stride(int F2, size_t tsize);
 // Interleave F in-place C2R outputs (padded real rows) at src into cell records
-// [cell][t2_record_stride(F)] at dst.
+// [cell][t2_record_stride(F, tsize)] at dst.
 cudaError_t run_t2_interleave(fkreg_plan_s* P, const int64_t* dims, int F, const void* src,
                               void* dst, cudaStream_t st);
 

@@ -417,8 +417,8 @@ struct GroupCtx {
 // Phase B of one pass: lane = sample (valid when lane < cnt).  Solves on pass 0,
 // then forms mhat for this pass's responses / probes and accumulates.  FP32
 // runs solve p <= 3 with the compensated FP32 closed forms, everything else
-// goes through FP64.
-template <typename T>
+// goes through FP64.  ORD: the order where the kernel knows it (else -1).
+template <typename T, int D, int ORD = -1>
 __device__ __forceinline__ void finish_pass(const GroupCtx& c, const MonoTab& mono, const BwDev& B,
                                             const T* my, int pass, int q_done, int q_in, int lane,
                                             bool valid, int64_t n, const T* cvp, int64_t cstride,
@@ -445,15 +445,14 @@ __device__ __forceinline__ void finish_pass(const GroupCtx& c, const MonoTab& mo
     } else {
       double a[kMaxP] = {0, 0, 0, 0};
       if (valid) {
-        double sv[kMaxMono];
+        constexpr int NSM = mono_count(D, D < 3 ? 4 : 2);  // s-fields of the highest order
+        double sv[NSM];
 #pragma unroll
-        for (int k = 0; k < kMaxMono; ++k) sv[k] = k < c.ns ? double(my[k]) : 0.0;
-        if (c.order == 0) {
-          ok = sv[0] > 0.0;
-          a[0] = ok ? 1.0 / sv[0] : 0.0;
-        } else {
-          ok = lpr_weights_fast(mono, c.p, sv, B.sigma, isg, a);
-        }
+        for (int k = 0; k < NSM; ++k) sv[k] = k < c.ns ? double(my[k]) : 0.0;
+        if constexpr (ORD >= 0)
+          ok = lpr_weights<D, ORD>(sv, isg, a);
+        else
+          ok = lpr_weights_order<D>(c.order, sv, isg, a);
       }
 #pragma unroll
       for (int k = 0; k < kMaxP; ++k) af[k] = (ok && k < c.p) ? T(a[k]) * tsc[k] : T(0);

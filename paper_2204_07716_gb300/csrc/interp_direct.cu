@@ -407,7 +407,7 @@ cudaError_t run_interp_direct(fkreg_plan_s* P, int b, int n_rhs_real, int n_prob
   if (P->prec != FKREG_F32 || P->geo.w != 7 || D > 2 || F2 > 64 || P->n == 0) return cudaSuccess;
   if (!vout && P->order > 1) return cudaSuccess;
   const BwDev& B = P->bw[b];
-  const int rec = t2_record_stride(F2);
+  const int rec = t2_record_stride(F2, sizeof(float));
   const int wm0 = tma_window(P->geo, B, 0);
   const int wm1 = D > 1 ? tma_window(P->geo, B, 1) : 1;
   if (wm0 > B.nf[0] || (D > 1 && wm1 > B.nf[1])) return cudaSuccess;

@@ -204,7 +204,7 @@ cudaError_t run_interp_global_lane(fkreg_plan_s* P, int b, int n_rhs_real, int n
   if (P->prec != FKREG_F32 || P->geo.w != 7 || P->d != 3 || F2 > 64 || P->n == 0)
     return cudaSuccess;
   if (!vout && P->order != 0) return cudaSuccess;
-  const int rec = t2_record_stride(F2);
+  const int rec = t2_record_stride(F2, sizeof(float));
   const int cst = vout ? 1 : ((n_rhs_real + n_probes) | 1);
   const size_t smem = sizeof(double) * size_t(kGWarps) * nacc +
                       sizeof(float) * size_t(kGWarps) * 32 * cst;

@@ -114,6 +114,7 @@ static void gauss_legendre(int n, std::vector<double>* x, std::vector<double>* w
   }
 }
 
+
 void spread_phihat(int kind, int w, double beta, int64_t nf, int64_t nk, double* out) {
   // phi is even: phihat(k) = 2 * integral_0^{w/2} phi(z) cos(2 pi k z / nf) dz.
   // The ES kernel has a square-root edge, so use many nodes.
@@ -228,6 +229,7 @@ static fkreg_status compute_geometry_direct(const fkreg_opts* o, fkreg_geometry*
     B.kr2 = gcut ? r2 : 0.0;
     for (int j = 0; j < 3; ++j) {
       B.sigma[j] = j < d ? std::sqrt(r2 * Hb[j * d + j]) : 1.0;
+      B.isigma[j] = 1.0 / B.sigma[j];
       B.K[j] = 1;
       B.nf[j] = j < d ? o->grid_n[j] : 1;
     }
@@ -380,6 +382,7 @@ fkreg_status compute_geometry(const fkreg_opts* o, fkreg_geometry* g, std::strin
     B.k0 = 1.0 / std::sqrt(std::pow(2.0 * M_PI, d) * det[b]);
     for (int j = 0; j < d; ++j) {
       B.sigma[j] = std::sqrt(Hb[j * d + j]);
+      B.isigma[j] = 1.0 / B.sigma[j];
       const double xi = xi_fac * std::sqrt(Hinv[size_t(b) * d * d + j * d + j]);
       int64_t half = int64_t(std::ceil(xi * g->period[j])) + 1;
       int64_t K = std::max<int64_t>(4, 2 * half);
@@ -392,6 +395,7 @@ fkreg_status compute_geometry(const fkreg_opts* o, fkreg_geometry* g, std::strin
       B.K[j] = 1;
       B.nf[j] = 1;
       B.sigma[j] = 1;
+      B.isigma[j] = 1;
     }
   }
   for (int j = 0; j < d; ++j) {

@@ -3,9 +3,10 @@
 // At every grid point the s- and t-fields give the normal equations
 // S(g) beta = t(g) of eqs. 3 / 11 (S_ab = s_(a+b)).  They are assembled in
 // FP64 in the scaled basis u = diag(sigma)^-1 (x_i - g), which leaves the
-// intercept unchanged, solved in closed form (p <= 3) or by Gaussian
-// elimination with partial pivoting (p = 4), and mhat = e_1^T S^-1 t.  Grid points whose density s_0 is below
-// mask_rho * max s_0 are masked (NaN estimate, mask 0).
+// intercept unchanged, solved in closed form (local linear in 1-D and 2-D) or by
+// Gaussian elimination with partial pivoting, and mhat = e_1^T S^-1 t.  Grid
+// points whose density s_0 is below mask_rho * max s_0 are masked (NaN
+// estimate, mask 0).
 #include <cuda_runtime.h>
 
 #include "device_common.cuh"
@@ -68,68 +69,70 @@ struct GridOut {
   double* avec;       // [n_bw][p][M] a_k / tscale_k (NaN where masked), or null
 };
 
-template <typename T>
-__global__ void grid_solve_kernel(GeoDev g, MonoTab mono, const BwDev* __restrict__ bwt,
-                                  int bw_first, int bw_count, int order, int64_t Mtot,
-                                  const T* __restrict__ field, int fgrid, int64_t lcells,
-                                  int nrhs_fields, const T* __restrict__ smax, double rho,
-                                  GridOut out) {
+// Thread per grid point, the system known at compile time (D, ORD): S stays in
+// registers, the scales 1 / sigma^g are formed once per point instead of one
+// FP64 division per response and unknown.  Bound by the FP64 pipe (two lanes
+// per SM and clock): 2-D local linear has some 50 FP64 instructions a point,
+// 2-D local quadratic some 250.
+template <typename T, int D, int ORD>
+__global__ void grid_solve_kernel(GeoDev g, const BwDev* __restrict__ bwt, int bw_first,
+                                  int bw_count, int64_t Mtot, const T* __restrict__ field,
+                                  int fgrid, int64_t lcells, int nrhs_fields,
+                                  const T* __restrict__ smax, double rho, GridOut out) {
+  constexpr int NS = mono_count(D, 2 * ORD), NT = mono_count(D, ORD);
   const int64_t gid = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (gid >= Mtot * bw_count) return;
   const int64_t m = gid % Mtot;
   const int bb = int(gid / Mtot);
   const int b = bw_first + bb;
   const BwDev& B = bwt[b];
-  int64_t rem = m, lidx = 0, mi[3];
-  for (int a = 2; a >= 0; --a) {
+  int64_t rem = m, lidx = 0, mi[3] = {0, 0, 0};
+#pragma unroll
+  for (int a = D - 1; a >= 0; --a) {
     mi[a] = rem % g.M[a];
     rem /= g.M[a];
   }
-  for (int a = 0; a < 3; ++a) lidx = lidx * g.L[a] + mi[a];
+#pragma unroll
+  for (int a = 0; a < D; ++a) lidx = lidx * g.L[a] + mi[a];
   if (!in_range(g.errw, kSiteSolveField, lidx, lcells)) return;
   const T* f0 = field + int64_t(bb) * fgrid * lcells + lidx;
-  const int ns = mono.n, nt = mono.nt;
-  double s[kMaxMono];
-  for (int k = 0; k < ns; ++k) s[k] = double(f0[int64_t(k) * lcells]);
-  const int p = nt;
-  double a[kMaxP] = {0, 0, 0, 0};
+  double s[NS], a[NT], its[NT];
+#pragma unroll
+  for (int k = 0; k < NS; ++k) s[k] = double(f0[int64_t(k) * lcells]);
+#pragma unroll
+  for (int k = 0; k < NT; ++k) a[k] = 0.0;
+  lpr_iscale<D, ORD>(B.isigma, its);
   bool ok = (s[0] > 0.0) && (s[0] >= rho * double(smax[bb]));
-  if (ok) {
-    if (order == 0)
-      a[0] = 1.0 / s[0];
-    else
-    {
-      const double isg[3] = {1.0 / B.sigma[0], 1.0 / B.sigma[1], 1.0 / B.sigma[2]};
-      ok = lpr_weights_fast(mono, p, s, B.sigma, isg, a);
-    }
+  if (ok) ok = lpr_weights<D, ORD>(s, B.isigma, a);
+  const double dnan = __longlong_as_double(0x7ff8000000000000LL);
+  const T nan = T(dnan);
+#pragma unroll
+  for (int k = 0; k < NT; ++k) {
+    a[k] *= its[k];
+    if (out.avec) out.avec[(int64_t(b) * NT + k) * Mtot + m] = ok ? a[k] : dnan;
   }
-  const T nan = T(__longlong_as_double(0x7ff8000000000000LL));
-  if (out.avec)
-    for (int k = 0; k < p; ++k)
-      out.avec[(int64_t(b) * p + k) * Mtot + m] =
-          ok ? a[k] / tscale(mono, k, B.sigma) : __longlong_as_double(0x7ff8000000000000LL);
   const int mult = out.cplx ? 2 : 1;
-  for (int q = 0; q < nrhs_fields; ++q) {
-    double mh = 0.0;
-    const T* tq = f0 + int64_t(ns + q * nt) * lcells;
-    for (int k = 0; k < p; ++k) mh += a[k] * double(tq[int64_t(k) * lcells]) / tscale(mono, k, B.sigma);
-    if (out.mhat) {
+  if (out.mhat)
+    for (int q = 0; q < nrhs_fields; ++q) {
+      double mh = 0.0;
+      const T* tq = f0 + int64_t(NS + q * NT) * lcells;
+#pragma unroll
+      for (int k = 0; k < NT; ++k) mh += a[k] * double(tq[int64_t(k) * lcells]);
       const int r = q / mult, part = q % mult;
       T* o = static_cast<T*>(out.mhat);
       o[((int64_t(b) * out.n_rhs_out + r) * Mtot + m) * mult + part] = ok ? T(mh) : nan;
     }
-  }
   if (out.mask) out.mask[int64_t(b) * Mtot + m] = ok ? 1 : 0;
   if (out.moments) {
     T* o = static_cast<T*>(out.moments);
-    const int64_t slice = int64_t(ns + nrhs_fields * nt) * Mtot;
+    const int64_t slice = int64_t(NS + nrhs_fields * NT) * Mtot;
     T* ob = o + int64_t(b) * slice;
-    for (int k = 0; k < ns; ++k) ob[int64_t(k) * Mtot + m] = f0[int64_t(k) * lcells];
+    for (int k = 0; k < NS; ++k) ob[int64_t(k) * Mtot + m] = f0[int64_t(k) * lcells];
     for (int q = 0; q < nrhs_fields; ++q) {
       const int r = q / mult, part = q % mult;
-      for (int k = 0; k < nt; ++k)
-        ob[int64_t(ns) * Mtot + ((int64_t(r) * nt + k) * Mtot + m) * mult + part] =
-            f0[int64_t(ns + q * nt + k) * lcells];
+      for (int k = 0; k < NT; ++k)
+        ob[int64_t(NS) * Mtot + ((int64_t(r) * NT + k) * Mtot + m) * mult + part] =
+            f0[int64_t(NS + q * NT + k) * lcells];
     }
   }
 }
@@ -208,11 +211,17 @@ cudaError_t launch_grid_solve(fkreg_plan_s* P, int bw_first, int bw_count, int n
     go.cplx = P->o.y_complex;
     go.n_rhs_out = P->nrhs;
   }
-  grid_solve_kernel<T><<<blocks, 256, 0, st>>>(g, P->mono, wsp<BwDev>(P, P->r_bw), bw_first,
-                                               bw_count, P->order, Mtot, field, fgrid, lcells,
-                                               nrhs_fields, smax, rho, go);
   P->launches += 2;
-  return cudaGetLastError();
+#define FK_GS(DD, OO)                                                                        \
+  if (P->d == DD && P->order == OO) {                                                        \
+    grid_solve_kernel<T, DD, OO><<<blocks, 256, 0, st>>>(g, wsp<BwDev>(P, P->r_bw), bw_first, \
+                                                         bw_count, Mtot, field, fgrid,       \
+                                                         lcells, nrhs_fields, smax, rho, go); \
+    return cudaGetLastError();                                                               \
+  }
+  FK_GS(1, 0) FK_GS(1, 1) FK_GS(1, 2) FK_GS(2, 0) FK_GS(2, 1) FK_GS(2, 2) FK_GS(3, 0) FK_GS(3, 1)
+#undef FK_GS
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace

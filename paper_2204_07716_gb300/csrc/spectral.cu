@@ -991,7 +991,7 @@ cudaError_t run_t2_interleave(fkreg_plan_s* P, const int64_t* dims, int F, const
   const int64_t nlast = dims[D - 1];
   const int64_t row_pitch = 2 * (nlast / 2 + 1);
   const int64_t fdist = rows * row_pitch;
-  const int rec = t2_record_stride(F);
+  const int rec = t2_record_stride(F, P->tsize);
   if (cells == 0 || F == 0) return cudaSuccess;
   const unsigned blocks = unsigned((cells + 31) / 32);
   const size_t smem = size_t(F) * 33 * P->tsize;

@@ -321,9 +321,10 @@ spread_run_kernel(GeoDev g, int64_t n, const T* __restrict__ xs, const T* __rest
         const T f0 = ceil(u - halfw);
         const int l = int(int64_t(f0) - o[j]);
         org = j == 0 ? l : org * W3[1] + l;
-        const T off = f0 - u;
+        T v[W];
+        phi_row<W>(g.skind, beta, f0 - u, v);
 #pragma unroll
-        for (int t = 0; t < W; ++t) phi_rows[lane * PS + j * W + t] = phi<T>(g.skind, W, beta, off + T(t));
+        for (int t = 0; t < W; ++t) phi_rows[lane * PS + j * W + t] = v[t];
       }
       org_row[lane] = org;
 #pragma unroll
