@@ -17,7 +17,10 @@ namespace fk {
 constexpr int kMaxD = 3;
 constexpr int kMaxMono = 35;     // monomials of degree <= 4 in 3-D (s-fields of local quadratic)
 constexpr int kMaxP = 10;        // unknowns of the local-quadratic system in 3-D
-constexpr int kSubMax = 1024;    // samples per spreading sub-problem
+// Samples per sub-problem (a run of one bin's samples that one block takes in
+// the spreading and the staged gathers): GeoDev::sub_max, between these.
+constexpr int kSubMin = 256;
+constexpr int kSubMax = 1024;
 constexpr int kRadixBits = 8;
 constexpr int kSortTileKeys = 4096;  // keys per radix-sort tile (one block)
 constexpr uint32_t kDefaultWaitLimit = 1u << 22;  // polls of a staged-window wait
@@ -42,6 +45,7 @@ struct GeoDev {
   int64_t nbins[3];
   int kbits;        // within-bin bits of the sort key (see key_local_bits)
   int kern;         // regression kernel: FKREG_KERNEL_GAUSSIAN (NUFFT) or a compact one (direct)
+  uint32_t sub_max;     // samples per sub-problem (sub_problem_size)
   uint32_t wait_limit;  // polls of a staged-window wait before it gives up (fkreg_set_wait_limit)
   int* errw;            // the plan's error word (errw[0] bits kErr*; errw[1..3] the first
                         // failed bounds check of a checked build: site, index low, high)
@@ -70,6 +74,22 @@ inline int key_local_bits(int d, const int64_t* tile, const int64_t* nbins) {
   while ((int64_t(1) << lb) < cells) ++lb;
   while ((int64_t(1) << bb) < bins) ++bb;
   return bb + lb <= 32 ? lb : 0;
+}
+
+// Sub-problem size of a plan for up to max_n samples in nbins bins.  Where the
+// bins are fewer than two per SM they are split into about four sub-problems
+// per SM, so that a small problem fills the GPU (10,000 1-D samples in one
+// bin: 10 blocks of 1024 before, 40 of 256 now, a group of 32 for each warp).  More
+// bins than that give blocks enough by themselves, and every further split
+// pays for one more tile flush (16 strengths of a 24 x 24 tile against some
+// hundred samples: the GCV backward of 89,787 samples in 250 bins ran 10 % slower
+// with 160 than with 1024).  FP64 2-D blocks are long (the FP64 pipe) against
+// their flush: there the split also evens out the last wave.
+inline uint32_t sub_problem_size(int d, bool f64, int64_t nbins, int64_t max_n, int sm_count) {
+  const int64_t sms = sm_count < 1 ? 1 : sm_count;
+  if (d > 2 || (nbins >= 2 * sms && !f64)) return kSubMax;
+  const int64_t per = (max_n / (4 * sms) + 31) / 32 * 32;
+  return uint32_t(per < kSubMin ? kSubMin : (per > kSubMax ? kSubMax : per));
 }
 
 // One bandwidth, stored in the workspace (device reads it).

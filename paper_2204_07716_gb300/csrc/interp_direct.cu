@@ -132,7 +132,7 @@ interp_direct_kernel(GeoDev g, const BwDev* __restrict__ bwt, int b, int64_t n,
     int o0, o1;
     window_of(k, o0, o1);
     const uint32_t first = sub_first[k];
-    const uint32_t last = min(first + uint32_t(kSubMax), bin_start[sub_bin[k] + 1]);
+    const uint32_t last = min(first + g.sub_max, bin_start[sub_bin[k] + 1]);
     const int ngr = int((last - first + 31) / 32);
     // groups are claimed one ahead: the next group's coordinates load while
     // this one is processed

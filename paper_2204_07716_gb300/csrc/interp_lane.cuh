@@ -270,7 +270,7 @@ interp_lane_kernel(GeoDev g, MonoTab mono, LaneArgs a, const BwDev* __restrict__
   for (uint32_t k = blockIdx.x; k < nsub; k += gridDim.x) {
     const uint32_t bin = sub_bin[k];
     const uint32_t first = sub_first[k];
-    const uint32_t last = min(first + uint32_t(kSubMax), bin_start[bin + 1]);
+    const uint32_t last = min(first + g.sub_max, bin_start[bin + 1]);
     const int o0 = int(floor(double(int64_t(bin) / g.nbins[1] * g.tile[0]) * r0)) - g.pad - a.lo_slack;
     const int o1 = int(floor(double(int64_t(bin) % g.nbins[1] * g.tile[1]) * r1)) - g.pad - a.lo_slack;
     if (threadIdx.x == 0)

@@ -166,13 +166,14 @@ keys_tiles_kernel(GeoDev g, int64_t n, int64_t nbins, int64_t ntiles, const T* _
     if (hb[b]) atomicAdd(&counts[b], hb[b]);
 }
 
-// Bin starts and spreading sub-problems (at most kSubMax samples each) from
+// Bin starts and spreading sub-problems (at most sub_max samples each) from
 // the bin counts, by one block of kDigitScanWarps warps: each thread owns a
 // contiguous chunk of bins, the block scans the chunk totals of samples and
 // sub-problems, and each thread writes its bins' starts and sub-problems.
 struct BinsArgs {
   const uint32_t* counts;
   int64_t nbins;
+  uint32_t sub_max;
   uint32_t* bin_start;  // [nbins + 1]
   uint32_t* sub_start;  // [nbins + 1]
   uint32_t* sub_bin;
@@ -189,7 +190,7 @@ __device__ void bins_block(const BinsArgs& a) {
   for (int64_t b = b0; b < b1; ++b) {
     const uint32_t c = a.counts[b];
     tc += c;
-    ts += (c + kSubMax - 1) / kSubMax;
+    ts += (c + a.sub_max - 1) / a.sub_max;
   }
   uint32_t ic = tc, is = ts;
   for (int o = 1; o < 32; o <<= 1) {
@@ -215,12 +216,12 @@ __device__ void bins_block(const BinsArgs& a) {
     tots += ws[w];
   }
   for (int64_t b = b0; b < b1; ++b) {
-    const uint32_t c = a.counts[b], ns = (c + kSubMax - 1) / kSubMax;
+    const uint32_t c = a.counts[b], ns = (c + a.sub_max - 1) / a.sub_max;
     a.bin_start[b] = rc;
     a.sub_start[b] = rs;
     for (uint32_t k = 0; k < ns; ++k) {
       a.sub_bin[rs + k] = uint32_t(b);
-      a.sub_first[rs + k] = rc + k * kSubMax;
+      a.sub_first[rs + k] = rc + k * a.sub_max;
     }
     rc += c;
     rs += ns;
@@ -603,13 +604,13 @@ __global__ void gather_coords_kernel(GeoDev g, int64_t n, const T* __restrict__ 
 }
 
 __global__ void nsub_kernel(const uint32_t* __restrict__ counts, int64_t nbins,
-                            uint32_t* __restrict__ nsub) {
+                            uint32_t sub_max, uint32_t* __restrict__ nsub) {
   const int64_t b = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (b >= nbins) return;
-  nsub[b] = (counts[b] + kSubMax - 1) / kSubMax;
+  nsub[b] = (counts[b] + sub_max - 1) / sub_max;
 }
 
-__global__ void fill_sub_kernel(const uint32_t* __restrict__ bin_start, int64_t nbins,
+__global__ void fill_sub_kernel(const uint32_t* __restrict__ bin_start, int64_t nbins, uint32_t sub_max,
                                 const uint32_t* __restrict__ sub_start,
                                 uint32_t* __restrict__ sub_bin, uint32_t* __restrict__ sub_first) {
   const int64_t b = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -617,7 +618,7 @@ __global__ void fill_sub_kernel(const uint32_t* __restrict__ bin_start, int64_t 
   const uint32_t s0 = sub_start[b], s1 = sub_start[b + 1];
   for (uint32_t k = s0; k < s1; ++k) {
     sub_bin[k] = uint32_t(b);
-    sub_first[k] = bin_start[b] + (k - s0) * kSubMax;
+    sub_first[k] = bin_start[b] + (k - s0) * sub_max;
   }
 }
 
@@ -725,6 +726,7 @@ cudaError_t run_sort_fused(fkreg_plan_s* P, int64_t n, const T* x, int passes, i
   constexpr size_t sm = radix_down_smem<B>();
   const BinsArgs bins{counts,
                       nbins,
+                      g.sub_max,
                       wsp<uint32_t>(P, P->r_binstart),
                       wsp<uint32_t>(P, P->r_substart),
                       wsp<uint32_t>(P, P->r_subbin),
@@ -833,14 +835,14 @@ cudaError_t run_sort(fkreg_plan_s* P, int64_t n, const void* x, cudaStream_t s) 
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     P->launches += 1;
   }
-  // spreading sub-problems: at most kSubMax samples each
+  // spreading sub-problems: at most sub_max samples each
   uint32_t* nsub = wsp<uint32_t>(P, P->r_nsub);
   uint32_t* sstart = wsp<uint32_t>(P, P->r_substart);
   const unsigned bb = unsigned((nbins + 255) / 256);
-  nsub_kernel<<<bb, 256, 0, s>>>(counts, nbins, nsub);
+  nsub_kernel<<<bb, 256, 0, s>>>(counts, nbins, g.sub_max, nsub);
   P->launches += 2;
   if ((e = exclusive_scan(nsub, sstart, nbins, scratch, s, &P->launches)) != cudaSuccess) return e;
-  fill_sub_kernel<<<bb, 256, 0, s>>>(bstart, nbins, sstart, wsp<uint32_t>(P, P->r_subbin),
+  fill_sub_kernel<<<bb, 256, 0, s>>>(bstart, nbins, g.sub_max, sstart, wsp<uint32_t>(P, P->r_subbin),
                                      wsp<uint32_t>(P, P->r_subfirst));
   return cudaGetLastError();
 }

@@ -1,7 +1,7 @@
 // Type-1 spreading (the gridding of Sec. 1.2, eqs. 16-17) and strength setup.
 //
 // fine_s[m] = sum_i c_{s,i} prod_j phi(m_j - u_ij),  u_ij = (x_ij - lo_j) nf_j / P_j,
-// periodic in m_j (mod nf_j).  One CTA owns one sub-problem: up to kSubMax
+// periodic in m_j (mod nf_j).  One CTA owns one sub-problem: up to sub_max
 // sorted samples of one bin, accumulated into a shared-memory copy of the
 // bin's tile plus a halo of ceil(w/2) cells per side; the CTA then adds the
 // tile to the fine grid in global memory with one atomic per non-zero cell.
@@ -59,7 +59,7 @@ spread_kernel(GeoDev g, int64_t n, const T* __restrict__ xs, const T* __restrict
   if (k >= *sub_total) return;
   const uint32_t b = sub_bin[k];
   const uint32_t first = sub_first[k];
-  const uint32_t last = min(first + uint32_t(kSubMax), bin_start[b + 1]);
+  const uint32_t last = min(first + g.sub_max, bin_start[b + 1]);
   int64_t bj[3] = {0, 0, 0};
   {
     int64_t rem = b;
@@ -246,7 +246,7 @@ spread_run_kernel(GeoDev g, int64_t n, const T* __restrict__ xs, const T* __rest
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t b = sub_bin[k];
   const uint32_t first = sub_first[k];
-  const uint32_t last = min(first + uint32_t(kSubMax), bin_start[b + 1]);
+  const uint32_t last = min(first + g.sub_max, bin_start[b + 1]);
   int64_t bj[2] = {0, 0};
   {
     int64_t rem = b;
