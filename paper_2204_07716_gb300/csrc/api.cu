@@ -235,6 +235,8 @@ fkreg_status fkreg_plan_create(const fkreg_opts* opts, int64_t max_n, fkreg_plan
   P->nrhs = opts->n_rhs;
   P->nrhs_real = opts->n_rhs * (opts->y_complex ? 2 : 1);
   P->max_probes = opts->max_probes;
+  if (P->prec == FKREG_F64 && P->g.w <= 2 * fk::kPhiTaps - 1)
+    fk::spread_phi_poly(P->geo.skind, P->geo.w, P->geo.beta, &P->poly);
   P->mono.n = P->ns;
   P->mono.nt = P->nt;
   fk::monomials(d, 2 * P->order, P->mono.e);

@@ -57,11 +57,50 @@ __device__ __forceinline__ float phi<float>(int kind, int w, float beta, float z
 }
 
 // All W kernel values phi(off + t), t = 0 .. W-1, of one axis (off is the first
-// cell's offset, in [-w/2, -w/2 + 1)).
-template <int W, typename T>
-__device__ __forceinline__ void phi_row(int skind, T beta, T off, T (&v)[W]) {
+// cell's offset, in [-w/2, -w/2 + 1)).  FP32: phi at each.  FP64: with
+// x = off + (W - 1)/2 in [-1/2, 1/2) the taps lie at x +- c, and each pair is
+// phi(x +- c) = E_c(x^2) +- x O_c(x^2) with polynomials of eight coefficients
+// fitted when the plan is made (PhiPoly), right to 2e-16 of the peak; the two
+// outermost taps, where the square root ends, are evaluated.  A pair costs 16
+// instructions on the FP64 pipe (one warp instruction per SM and 16 clocks)
+// where two square roots and exponentials take some 90.
+template <typename T>
+struct PhiTab {};  // FP32 needs no table
+template <>
+struct PhiTab<double> {
+  PhiPoly p;
+};
+template <int W>
+__device__ __forceinline__ void phi_row(const PhiTab<float>&, int skind, float beta, float off,
+                                        float (&v)[W]) {
 #pragma unroll
-  for (int t = 0; t < W; ++t) v[t] = phi<T>(skind, W, beta, off + T(t));
+  for (int t = 0; t < W; ++t) v[t] = phi<float>(skind, W, beta, off + float(t));
+}
+template <typename T>
+__device__ __noinline__ T phi_call(int skind, int w, T beta, T z) {
+  return phi<T>(skind, w, beta, z);
+}
+template <int W>
+__device__ __forceinline__ void phi_row(const PhiTab<double>& tab, int skind, double beta,
+                                        double off, double (&v)[W]) {
+  const double x = off + 0.5 * (W - 1), y = x * x;
+  v[0] = phi_call<double>(skind, W, beta, off);
+  v[W - 1] = phi_call<double>(skind, W, beta, off + (W - 1));
+#pragma unroll
+  for (int k = 1; k < (W + 1) / 2; ++k) {
+    double e = tab.p.e[k][kPhiTerms - 1], o = tab.p.o[k][kPhiTerms - 1];
+#pragma unroll
+    for (int j = kPhiTerms - 2; j >= 0; --j) {
+      e = fma(e, y, tab.p.e[k][j]);
+      if (2 * k != W - 1) o = fma(o, y, tab.p.o[k][j]);
+    }
+    if (2 * k == W - 1) {
+      v[k] = e;
+    } else {  // tap k lies at x - c, its mirror at x + c
+      v[k] = fma(-x, o, e);
+      v[W - 1 - k] = fma(x, o, e);
+    }
+  }
 }
 
 // Compile-time chain of the monomials of degree <= DEG in d = D variables, in

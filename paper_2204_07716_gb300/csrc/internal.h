@@ -25,6 +25,16 @@ constexpr int kRadixBits = 8;
 constexpr int kSortTileKeys = 4096;  // keys per radix-sort tile (one block)
 constexpr uint32_t kDefaultWaitLimit = 1u << 22;  // polls of a staged-window wait
 
+// Polynomials of the spreading kernel's inner taps (phi_row), tap k at distance
+// c = (w - 1)/2 - k from the centre: phi(x +- c) = E(x^2) +- x O(x^2) for
+// |x| <= 1/2.  FP64 plans of an instantiated width.
+constexpr int kPhiTerms = 8;
+constexpr int kPhiTaps = 7;
+struct PhiPoly {
+  double e[kPhiTaps][kPhiTerms];
+  double o[kPhiTaps][kPhiTerms];
+};
+
 // Geometry of the whole plan, passed to kernels by value.
 struct GeoDev {
   int d;
@@ -126,6 +136,7 @@ struct fkreg_plan_s {
   fkreg_geometry g{};
   fk::GeoDev geo{};
   fk::MonoTab mono{};
+  fk::PhiPoly poly{};           // FP64 plans
   int64_t max_n = 0;
   int d = 0, order = 0, prec = 0, ns = 0, nt = 0, p = 0;
   int nbw = 0, nrhs = 0, nrhs_real = 0, max_probes = 0;
@@ -194,6 +205,7 @@ fkreg_status compute_geometry(const fkreg_opts* o, fkreg_geometry* g, std::strin
                               std::vector<BwDev>* bw, std::vector<double>* tab,
                               int64_t phi1_off[3], GeoDev* geo);
 double spread_phi(int kind, int w, double beta, double z);
+void spread_phi_poly(int kind, int w, double beta, PhiPoly* out);
 void spread_phihat(int kind, int w, double beta, int64_t nf, int64_t nk, double* out);
 int nmono(int d, int deg);
 void monomials(int d, int deg, int (*e)[kMaxD]);

@@ -127,13 +127,13 @@ struct LeadAxes {
   int lane, skind;
   T beta;
   T off[D];
-  __device__ __forceinline__ void set(const T* o) {
+  __device__ __forceinline__ void set(const PhiTab<T>& tab, const T* o) {
 #pragma unroll
     for (int j = 0; j < D; ++j) off[j] = o[j];
 #pragma unroll
     for (int j = 0; j < lane_axes_parked<T, D>(); ++j) {
       T v[W];
-      phi_row<W>(skind, beta, o[j], v);
+      phi_row<W>(tab, skind, beta, o[j], v);
 #pragma unroll
       for (int t = 0; t < W; ++t) park[(j * W + t) * 32 + lane] = v[t];
     }
@@ -225,7 +225,7 @@ constexpr int kLaneWarps = 8;  // warps per block (upper bound)
 // and exits), then each warp takes groups of 32 samples.
 template <typename T, int W, int NU>
 __global__ void __launch_bounds__(kLaneWarps * 32)
-interp_lane_kernel(GeoDev g, MonoTab mono, LaneArgs a, const BwDev* __restrict__ bwt, int64_t n,
+interp_lane_kernel(GeoDev g, MonoTab mono, LaneArgs a, PhiTab<T> tab, const BwDev* __restrict__ bwt, int64_t n,
                    const T* __restrict__ xs, const T* __restrict__ str,
                    const uint32_t* __restrict__ perm, const T* __restrict__ fld,
                    T* __restrict__ mhat_at_x, double* __restrict__ part,
@@ -300,8 +300,8 @@ interp_lane_kernel(GeoDev g, MonoTab mono, LaneArgs a, const BwDev* __restrict__
                                       int64_t(l0 + W - 1) * a.pitch + int64_t(l1 + W) * a.rec - 1,
                                       int64_t(a.wm0) * a.pitch);
       T pl[W];
-      lead.set(off);
-      phi_row<W>(g.skind, beta, off[1], pl);
+      lead.set(tab, off);
+      phi_row<W>(tab, g.skind, beta, off[1], pl);
       const uint32_t orig = !vout && valid ? perm[s] : 0u;
       T af[kMaxP] = {T(0), T(0), T(0), T(0)};
       int q_done = 0, f_first = 0;
@@ -348,7 +348,7 @@ interp_lane_kernel(GeoDev g, MonoTab mono, LaneArgs a, const BwDev* __restrict__
 // ---- straight from the field grid ------------------------------------------
 template <typename T, int D, int W, int NU>
 __global__ void __launch_bounds__(kLaneWarps * 32)
-interp_global_kernel(GeoDev g, MonoTab mono, LaneArgs a, const BwDev* __restrict__ bwt, int64_t n,
+interp_global_kernel(GeoDev g, MonoTab mono, LaneArgs a, PhiTab<T> tab, const BwDev* __restrict__ bwt, int64_t n,
                      const T* __restrict__ xs, const T* __restrict__ str,
                      const uint32_t* __restrict__ perm, const T* __restrict__ fld,
                      T* __restrict__ mhat_at_x, double* __restrict__ part, T* __restrict__ vout) {
@@ -389,8 +389,8 @@ interp_global_kernel(GeoDev g, MonoTab mono, LaneArgs a, const BwDev* __restrict
 #pragma unroll
     for (int j = 0; j < D; ++j) i[j] = lane_window<T>(xs[int64_t(j) * n + sl], ih[j], halfw, off[j]);
     T pl[W];
-    lead.set(off);
-    phi_row<W>(g.skind, beta, off[D - 1], pl);
+    lead.set(tab, off);
+    phi_row<W>(tab, g.skind, beta, off[D - 1], pl);
     const uint32_t orig = !vout && valid ? perm[s] : 0u;
     T af[kMaxP] = {T(0), T(0), T(0), T(0)};
     int q_done = 0, f_first = 0;
@@ -431,6 +431,7 @@ struct LaneLaunch {
   T* mhat_at_x;
   T* vout;
   cudaStream_t st;
+  PhiTab<T> tab;
 };
 
 // shared memory of one warp, and warps per block that fit `budget` bytes,
@@ -465,7 +466,7 @@ cudaError_t launch_lane_staged(const LaneLaunch<T>& L, bool* launched) {
   if (e != cudaSuccess) return e;
   *launched = true;
   kern<<<unsigned(P->nblk_interp), nw * 32, smem, L.st>>>(
-      P->geo, P->mono, a, wsp<BwDev>(P, P->r_bw), P->n, wsp<T>(P, P->r_xs), wsp<T>(P, P->r_str),
+      P->geo, P->mono, a, L.tab, wsp<BwDev>(P, P->r_bw), P->n, wsp<T>(P, P->r_xs), wsp<T>(P, P->r_str),
       perm_ptr(P), wsp<T>(P, P->r_t2field), L.mhat_at_x, wsp<double>(P, P->r_part),
       wsp<uint32_t>(P, P->r_subbin), wsp<uint32_t>(P, P->r_subfirst),
       wsp<uint32_t>(P, P->r_binstart), wsp<uint32_t>(P, P->r_substart) + P->nbins_total, L.vout);
@@ -485,7 +486,7 @@ cudaError_t launch_lane_global(const LaneLaunch<T>& L) {
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
   kern<<<unsigned(P->nblk_interp), nw * 32, smem, L.st>>>(
-      P->geo, P->mono, L.a, wsp<BwDev>(P, P->r_bw), P->n, wsp<T>(P, P->r_xs), wsp<T>(P, P->r_str),
+      P->geo, P->mono, L.a, L.tab, wsp<BwDev>(P, P->r_bw), P->n, wsp<T>(P, P->r_xs), wsp<T>(P, P->r_str),
       perm_ptr(P), wsp<T>(P, P->r_t2field), L.mhat_at_x, wsp<double>(P, P->r_part), L.vout);
   P->launches += 1;
   return cudaGetLastError();

@@ -8,7 +8,7 @@ namespace fk {
 cudaError_t run_interp_lane_f64(fkreg_plan_s* P, int b, int n_rhs_real, int n_probes,
                                 void* mhat_at_x, cudaStream_t st, int nacc, int F2, void* vout,
                                 bool* launched) {
-  LaneLaunch<double> L{P, {}, static_cast<double*>(mhat_at_x), static_cast<double*>(vout), st};
+  LaneLaunch<double> L{P, {}, static_cast<double*>(mhat_at_x), static_cast<double*>(vout), st, {P->poly}};
   L.a.b = b;
   L.a.order = P->order;
   L.a.rec = t2_record_stride(F2, sizeof(double));

@@ -114,6 +114,40 @@ static void gauss_legendre(int n, std::vector<double>* x, std::vector<double>* w
   }
 }
 
+// Fits of the inner taps' even and odd parts in y = x^2 by Newton
+// interpolation at Chebyshev nodes of [0, 1/4] (near minimax for these
+// smooth functions), expanded to monomials in extended precision.
+void spread_phi_poly(int kind, int w, double beta, PhiPoly* out) {
+  std::memset(out, 0, sizeof(*out));
+  using L = long double;
+  auto f = [&](L z) -> L {
+    if (kind == FKREG_SPREAD_GAUSS) return std::exp(-L(beta) * z * z);
+    const L t = 2.0L * z / L(w), a = 1.0L - t * t;
+    return a > 0 ? std::exp(L(beta) * (std::sqrt(a) - 1.0L)) : 0.0L;
+  };
+  const L pi = 3.14159265358979323846264338327950288L;
+  for (int k = 1; k < std::min((w + 1) / 2, kPhiTaps); ++k) {
+    const L c = L(w - 1) / 2 - L(k);
+    L y[kPhiTerms], d[2][kPhiTerms];
+    for (int j = 0; j < kPhiTerms; ++j) {
+      y[j] = 0.125L + 0.125L * std::cos(pi * (L(j) + 0.5L) / kPhiTerms);
+      const L x = std::sqrt(y[j]), hi = f(c + x), lo = f(c - x);
+      d[0][j] = (hi + lo) / 2;
+      d[1][j] = (hi - lo) / (2 * x);
+    }
+    for (int s = 0; s < 2; ++s) {
+      for (int m = 1; m < kPhiTerms; ++m)  // divided differences
+        for (int j = kPhiTerms - 1; j >= m; --j) d[s][j] = (d[s][j] - d[s][j - 1]) / (y[j] - y[j - m]);
+      L p[kPhiTerms] = {0};
+      for (int j = kPhiTerms - 1; j >= 0; --j) {  // p = p (y - y_j) + d_j
+        for (int m = kPhiTerms - 1; m > 0; --m) p[m] = p[m - 1] - y[j] * p[m];
+        p[0] = d[s][j] - y[j] * p[0];
+      }
+      for (int m = 0; m < kPhiTerms; ++m) (s == 0 ? out->e : out->o)[k][m] = double(p[m]);
+    }
+  }
+}
+
 
 void spread_phihat(int kind, int w, double beta, int64_t nf, int64_t nk, double* out) {
   // phi is even: phihat(k) = 2 * integral_0^{w/2} phi(z) cos(2 pi k z / nf) dz.

@@ -230,7 +230,8 @@ __global__ void __launch_bounds__(kSpreadThreads)
 spread_run_kernel(GeoDev g, int64_t n, const T* __restrict__ xs, const T* __restrict__ str,
                   int s0, const uint32_t* __restrict__ sub_bin,
                   const uint32_t* __restrict__ sub_first, const uint32_t* __restrict__ bin_start,
-                  const uint32_t* __restrict__ sub_total, T* __restrict__ fine) {
+                  const uint32_t* __restrict__ sub_total, T* __restrict__ fine,
+                  PhiTab<T> tab) {
   static_assert(D <= 2 && W > 0, "run spreading serves 1-D and 2-D with a fixed width");
   constexpr int NC = D == 1 ? W : W * W;      // window cells
   constexpr int CS = (NC + 31) / 32;          // cell slots per lane
@@ -322,7 +323,7 @@ spread_run_kernel(GeoDev g, int64_t n, const T* __restrict__ xs, const T* __rest
         const int l = int(int64_t(f0) - o[j]);
         org = j == 0 ? l : org * W3[1] + l;
         T v[W];
-        phi_row<W>(g.skind, beta, f0 - u, v);
+        phi_row<W>(tab, g.skind, beta, f0 - u, v);
 #pragma unroll
         for (int t = 0; t < W; ++t) phi_rows[lane * PS + j * W + t] = v[t];
       }
@@ -431,6 +432,14 @@ size_t spread_run_smem(const GeoDev& g) {
          size_t(kSpreadThreads) * sizeof(int);
 }
 
+template <typename T>
+PhiTab<T> phi_tab(const fkreg_plan_s* P) {
+  if constexpr (sizeof(T) == 8)
+    return {P->poly};
+  else
+    return {};
+}
+
 template <typename T, int D, int W, int CN>
 cudaError_t launch_spread_run(fkreg_plan_s* P, int s0, cudaStream_t st) {
   const GeoDev& g = P->geo;
@@ -444,7 +453,7 @@ cudaError_t launch_spread_run(fkreg_plan_s* P, int s0, cudaStream_t st) {
   spread_run_kernel<T, D, W, CN><<<grid, kSpreadThreads, smem, st>>>(
       g, P->n, wsp<T>(P, P->r_xs), wsp<T>(P, P->r_str), s0, wsp<uint32_t>(P, P->r_subbin),
       wsp<uint32_t>(P, P->r_subfirst), wsp<uint32_t>(P, P->r_binstart), sub_total,
-      wsp<T>(P, P->r_fine));
+      wsp<T>(P, P->r_fine), phi_tab<T>(P));
   P->launches += 1;
   return cudaGetLastError();
 }
