@@ -240,6 +240,18 @@ fkreg_status fkreg_plan_create(const fkreg_opts* opts, int64_t max_n, fkreg_plan
   P->mono.n = P->ns;
   P->mono.nt = P->nt;
   fk::monomials(d, 2 * P->order, P->mono.e);
+  if ((opts->flags & FKREG_WANT_BACKWARD) && P->order <= 1) {
+    fk::MonoTab& all = P->mono_all;
+    fk::MonoTab& x = P->mono_x;
+    all.n = fk::nmono(d, 2 * P->order + 1);
+    all.nt = fk::nmono(d, P->order + 1);
+    fk::monomials(d, 2 * P->order + 1, all.e);
+    x.n = x.toff = all.n - P->ns;
+    x.nt = all.nt - P->nt;
+    for (int k = 0; k < x.n + x.nt; ++k)
+      std::memcpy(x.e[k], all.e[k < x.n ? P->ns + k : P->nt + k - x.n], sizeof(x.e[k]));
+    P->fxbwd = x.n + (1 + opts->max_probes) * x.nt;
+  }
   P->smax = 1 + P->nrhs_real + P->max_probes;
   P->f2max = P->ns + (P->nrhs_real + P->max_probes) * P->nt;
   P->fgrid = P->ns + P->nrhs_real * P->nt;
@@ -252,7 +264,7 @@ fkreg_status fkreg_plan_create(const fkreg_opts* opts, int64_t max_n, fkreg_plan
   const int nout_grid = P->nrhs_real + (1 + P->nrhs_real) * opts->dim;
   const int strengths_total = P->smax + (P->backward ? P->f2bwd : 0);
   const int t2_fields =
-      std::max(P->f2max, P->backward ? std::max(std::max(P->f2bwd, nout_bwd), nout_grid) : 0);
+      std::max(P->f2max, P->backward ? std::max({P->f2bwd, P->fxbwd, nout_bwd, nout_grid}) : 0);
   if (P->nacc > 512) {
     delete P;
     return set_global_error(FKREG_ERR_UNSUPPORTED, "n_rhs (real parts) + 2 max_probes must be <= 511");
@@ -343,10 +355,10 @@ fkreg_status fkreg_plan_create(const fkreg_opts* opts, int64_t max_n, fkreg_plan
     L.take(P->r_gmask, size_t(P->nbw) * mtot);
     L.take(P->r_gadj, T * size_t(P->ns + P->nrhs_real * P->nt) * l_cells);
     L.take(P->r_gpart, 8 * 3 * size_t(gblk));
-    L.take(P->r_bV, T * size_t(1 + 2 * d) * std::max(std::max(P->f2bwd, nout_bwd), nout_grid) * nn);
+    // the values and the extra moments, then the gathered adjoint fields
+    L.take(P->r_bV, T * size_t(std::max({P->f2bwd + P->fxbwd, nout_bwd, nout_grid})) * nn);
     L.take(P->r_bdx, T * size_t(d + 1) * nn);
-    L.take(P->r_bsc, 8 * 16);
-    L.take(P->r_bpart, 8 * 3 * size_t((nn + 255) / 256 + 1));
+    L.take(P->r_bsc, 8 * (16 + 1 + size_t(P->max_probes)));
   }
   // cuFFT plans for the standard passes (work sizes decide the reserved area)
   if (!P->direct) {
@@ -391,6 +403,7 @@ fkreg_status fkreg_plan_create(const fkreg_opts* opts, int64_t max_n, fkreg_plan
       if (P->max_probes > 0) bts.push_back(P->f2max);
       if (P->backward) {
         bts.push_back(P->f2bwd);
+        if (P->fxbwd > 0) bts.push_back(P->fxbwd);
         bts.push_back(nout_bwd);
         bts.push_back(nout_grid);
       }
@@ -497,13 +510,13 @@ namespace {
 
 fkreg_status exec_fft(fkreg_plan_s* P, int kind, const int64_t* dims, int batch, void* in, void* out,
                       cudaStream_t s) {
+  const bool fwd = kind == 0 || kind == 3;
   cufftHandle h;
   fkreg_status st = fk::fft_get(P, kind, dims, batch, &h);
   if (st != FKREG_OK) return st;
   if (cufftSetStream(h, s) != CUFFT_SUCCESS) return plan_err(P, FKREG_ERR_CUFFT, "cufftSetStream failed");
   cufftResult r;
   void* dst = kind == 2 ? in : out;  // kind 2 runs in place, then interleaves into out
-  const bool fwd = kind == 0 || kind == 3;
   if (P->prec == FKREG_F32) {
     r = fwd ? cufftExecR2C(h, static_cast<cufftReal*>(in), static_cast<cufftComplex*>(dst))
             : cufftExecC2R(h, static_cast<cufftComplex*>(in), static_cast<cufftReal*>(dst));
@@ -530,8 +543,11 @@ fkreg_status exec_fft(fkreg_plan_s* P, int kind, const int64_t* dims, int batch,
     if (_s != FKREG_OK) return _s;      \
   } while (0)
 
+// only_b >= 0: the at-sample pass of that bandwidth alone, with its field values
+// kept at `keep` (the backward).
 fkreg_status pipeline(fkreg_plan_s* P, const void* y, int n_probes, uint64_t seed, const void* probes,
-                      const fkreg_outputs* out, bool want_df, cudaStream_t s) {
+                      const fkreg_outputs* out, bool want_df, cudaStream_t s, int only_b = -1,
+                      void* keep = nullptr) {
   if (!P->ws) return plan_err(P, FKREG_ERR_STATE, "fkreg_set_workspace must come first");
   if (!P->points_set) return plan_err(P, FKREG_ERR_STATE, "fkreg_set_points must come first");
   if (P->n > 0 && !y) return plan_err(P, FKREG_ERR_INVALID_ARG, "y is NULL");
@@ -564,7 +580,8 @@ fkreg_status pipeline(fkreg_plan_s* P, const void* y, int n_probes, uint64_t see
     if (want_df || n_probes > 0 || (out && (out->mhat_at_x || out->rss))) {
       for (int b = 0; b < P->nbw; ++b) {
         FK_STAGE(FKREG_STAGE_INTERP);
-        FK_CHECK(fk::run_interp(P, b, P->nrhs_real, n_probes, y, out ? out->mhat_at_x : nullptr, s),
+        FK_CHECK(fk::run_interp(P, b, P->nrhs_real, n_probes, out ? out->mhat_at_x : nullptr,
+                                nullptr, s),
                  "direct sums at the samples");
       }
       FK_STAGE(FKREG_STAGE_FINALIZE);
@@ -626,10 +643,11 @@ fkreg_status pipeline(fkreg_plan_s* P, const void* y, int n_probes, uint64_t see
   if (at) {
     const int n_rhs_str = P->nrhs_real + n_probes;
     const int f2 = P->ns + n_rhs_str * P->nt;
-    for (int b = 0; b < P->nbw; ++b) {
+    const int b0 = only_b < 0 ? 0 : only_b, b1 = only_b < 0 ? P->nbw : only_b + 1;
+    for (int b = b0; b < b1; ++b) {
       {
         FK_STAGE(FKREG_STAGE_KMUL_T2);
-        FK_CHECK(fk::run_kmul_t2(P, b, 0, 1, n_rhs_str, s), "kmul type-2");
+        FK_CHECK(fk::run_kmul_t2(P, b, P->mono, 0, 1, n_rhs_str, s), "kmul type-2");
       }
       {
         FK_STAGE(FKREG_STAGE_FFT_T2);
@@ -637,7 +655,8 @@ fkreg_status pipeline(fkreg_plan_s* P, const void* y, int n_probes, uint64_t see
       }
       {
         FK_STAGE(FKREG_STAGE_INTERP);
-        FK_CHECK(fk::run_interp(P, b, P->nrhs_real, n_probes, y, out ? out->mhat_at_x : nullptr, s),
+        FK_CHECK(fk::run_interp(P, b, P->nrhs_real, n_probes, out ? out->mhat_at_x : nullptr, keep,
+                                s),
                  "interpolation");
       }
     }
@@ -691,7 +710,7 @@ fkreg_status fkreg_backward(fkreg_plan P, const void* y, int n_probes, uint64_t 
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   fkreg_outputs out{};
-  FK_STATUS(pipeline(P, y, n_probes, seed, probes, &out, true, s));
+  FK_STATUS(pipeline(P, y, n_probes, seed, probes, &out, true, s, b, P->ws + P->r_bV.off));
   if (P->n == 0) return FKREG_OK;
   const int d = P->d;
   const int R = 1 + n_probes;
@@ -702,24 +721,27 @@ fkreg_status fkreg_backward(fkreg_plan P, const void* y, int n_probes, uint64_t 
   const int64_t nf_cells = full_cells(P->g.nf, d), nf_half = half_cells(P->g.nf, d);
   FK_STAGE(FKREG_STAGE_BACKWARD);
   FK_CHECK(fk::run_loss_scalars(P, b, n_probes, s), "loss scalars");
-  // values, evaluation-point gradients, bandwidth derivatives of the fields
-  for (int mode = 0; mode < 1 + 2 * d; ++mode) {
-    const int kind = mode == 0 ? 0 : (mode <= d ? 1 : 2);
-    const int axis = mode == 0 ? 0 : (mode <= d ? mode - 1 : mode - 1 - d);
-    FK_CHECK(fk::run_kmul_t2_mode(P, b, 0, 1, R, kind, axis, s), "derivative spectra");
-    FK_STATUS(exec_fft(P, 2, P->bw[b].nf, F2, P->ws + P->r_t2spec.off, P->ws + P->r_t2field.off, s));
-    FK_CHECK(fk::run_gather_fields(P, b, F2, P->ws + P->r_bV.off + T * size_t(mode) * F2 * n, s),
-             "gather fields");
-  }
+  // The field values at the samples were kept by the forward pass.  Their
+  // gradients in the evaluation point are moments one degree higher (adjoint
+  // kernels below): one more set of fx fields instead of d sets of F2.
+  const int fx = P->mono_x.n + R * P->mono_x.nt;
+  FK_CHECK(fk::run_kmul_t2(P, b, P->mono_x, 0, 1, R, s), "moment spectra");
+  FK_STATUS(exec_fft(P, 2, P->bw[b].nf, fx, P->ws + P->r_t2spec.off, P->ws + P->r_t2field.off, s));
+  FK_CHECK(fk::run_gather_fields(P, b, fx, P->ws + P->r_bV.off + T * size_t(F2) * n, s),
+           "gather moments");
   FK_CHECK(fk::run_adjoint(P, b, n_probes, s), "adjoints");
   // adjoint spreading of Qbar (strengths smax .. smax + F2)
   FK_CHECK(fk::run_spread(P, P->smax, F2, s), "adjoint spread");
   FK_STATUS(exec_fft(P, 0, P->g.nf, F2, P->ws + P->r_fine.off + T * P->smax * nf_cells,
                      P->ws + P->r_spec.off + 2 * T * P->smax * nf_half, s));
+  if (dlogh)
+    FK_CHECK(fk::run_dlogh_spread(P, b, R, P->smax,
+                                  reinterpret_cast<double*>(P->ws + P->r_gpart.off), dlogh, s),
+             "bandwidth gradient");
   FK_CHECK(fk::run_kmul_adj(P, b, P->smax, 1 + R, s), "adjoint spectra");
   FK_STATUS(exec_fft(P, 2, P->bw[b].nf, nout, P->ws + P->r_t2spec.off, P->ws + P->r_t2field.off, s));
   FK_CHECK(fk::run_gather_fields(P, b, nout, P->ws + P->r_bV.off, s), "gather adjoint fields");
-  FK_CHECK(fk::run_combine(P, n_probes, dy, dx, dlogh, s), "combine");
+  FK_CHECK(fk::run_combine(P, n_probes, dy, dx, s), "combine");
   if (gcv) {
     cudaError_t e = cudaMemcpyAsync(gcv, P->ws + P->r_bsc.off + 2 * sizeof(double), sizeof(double),
                                     cudaMemcpyDeviceToDevice, s);
@@ -899,7 +921,7 @@ fkreg_status fkreg_log_variance(fkreg_plan P, const void* y, const void* mhat_at
       }
       {
         FK_STAGE(FKREG_STAGE_INTERP);
-        FK_CHECK(fk::run_interp(P, b, R, 0, y, v_at_x, s), "direct sums at the samples");
+        FK_CHECK(fk::run_interp(P, b, R, 0, v_at_x, nullptr, s), "direct sums at the samples");
       }
       FK_STAGE(FKREG_STAGE_FINALIZE);
       FK_CHECK(fk::run_kappa_sigma2(P, b, y, mhat_at_x, v_at_x, v_grid, kappa, sigma2, s), "kappa");
@@ -935,7 +957,7 @@ fkreg_status fkreg_log_variance(fkreg_plan P, const void* y, const void* mhat_at
     // v at the samples: type-2 of the same fields
     {
       FK_STAGE(FKREG_STAGE_KMUL_T2);
-      FK_CHECK(fk::run_kmul_t2(P, b, 0, 1, R, s), "kmul type-2");
+      FK_CHECK(fk::run_kmul_t2(P, b, P->mono, 0, 1, R, s), "kmul type-2");
     }
     {
       FK_STAGE(FKREG_STAGE_FFT_T2);
@@ -943,7 +965,7 @@ fkreg_status fkreg_log_variance(fkreg_plan P, const void* y, const void* mhat_at
     }
     {
       FK_STAGE(FKREG_STAGE_INTERP);
-      FK_CHECK(fk::run_interp(P, b, R, 0, y, v_at_x, s), "interpolation");
+      FK_CHECK(fk::run_interp(P, b, R, 0, v_at_x, nullptr, s), "interpolation");
     }
     {
       FK_STAGE(FKREG_STAGE_FINALIZE);

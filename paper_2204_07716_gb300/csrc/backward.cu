@@ -10,13 +10,18 @@
 //   s-field g              : -sum_(a+b=g) a_a bbar_b  (bbar = sum_r g_r S^-1 t_r)
 // with g_y = -2 L_RSS (y_i - mhat_y), g_p = L_tr (N / Np) w_pi / (w_p^T w_p).
 // Then
-//   d/dlog sigma_j = sum_i Qbar_i . dQ_i/dlog sigma_j      (derivative fields at x_i)
-//   d/dx_i (target) = sum_f Qbar_(i,f) grad_q Q_f(x_i)      (gradient fields at x_i)
+//   d/dlog sigma_j = sum_i Qbar_i . dQ_i/dlog sigma_j      (a spectral inner product, spectral.cu)
+//   d/dx_i (target) = sum_f Qbar_(i,f) grad_q Q_f(x_i)      (fields at x_i, below)
 //   d/dx_j (source) = sum_c c_(c,j) sum_(f in c) sum_i Qbar_(i,f) grad w_f(x_j - x_i)
 //   d/dy_j          = 2 L_RSS (y_j - mhat_y(x_j)) + sum_(f in y) sum_i Qbar_(i,f) w_f(x_j - x_i)
 // The last two are NUFFT convolutions of the adjoints spread as strengths.
-// Field values at the samples come from the interpolation kernels' gather-only
-// mode (same bin-window staging as the forward pass).
+// For the Gaussian, d w_f / d z_d = f_d w_(f - e_d) - w_(f + e_d) / sigma_d^2, so the
+// gradient of a field in its evaluation point is
+//   dQ_f/dq_d = Q_(f + e_d) / sigma_d^2 - f_d Q_(f - e_d):
+// the moments of one more degree (37 more fields for 2-D local linear with
+// eleven strengths) stand for D sets of gradient fields (78).
+// Field values at the samples come from the forward pass, which keeps them,
+// and from the interpolation kernels' gather-only mode.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -34,6 +39,10 @@ constexpr int kE1Threads = 256;
 //   sc[0] = L_RSS = (1/N) / (1 - tr/N)^2
 //   sc[1] = L_tr * N / Np,  L_tr = 2 (RSS/N) / (N (1 - tr/N)^3)
 //   sc[2] = GCV
+// and for the FP32 adjoints the factors 2 L_RSS and sc[1] / w_p^T w_p as sums of
+// two floats (fac, from sc[16]): near the minimum of GCV the gradient in log h is
+// a small difference of the residuals' and the trace's parts, and one rounding
+// of a factor to FP32 moved it by up to 2e-5.
 __global__ void loss_scalars_kernel(const double* __restrict__ sums, int b, int nacc, int n_probes,
                                     int64_t n, double* __restrict__ sc) {
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
@@ -47,26 +56,37 @@ __global__ void loss_scalars_kernel(const double* __restrict__ sums, int b, int 
   sc[0] = (1.0 / N) / (den * den);
   sc[1] = (2.0 * (rss / N) / (N * den * den * den)) * (N / n_probes);
   sc[2] = (rss / N) / (den * den);
+  float2* fac = reinterpret_cast<float2*>(sc + 16);
+  for (int r = 0; r <= n_probes; ++r) {
+    const double v = r == 0 ? 2.0 * sc[0] : sc[1] / sb[n_probes + r];
+    const float hi = float(v);
+    fac[r] = make_float2(hi, float(v - double(hi)));
+  }
 }
 
-// Per-sample adjoints.  V holds (1 + 2D) blocks of F2 fields: values, the D
-// gradient fields and the D bandwidth-derivative fields.  Writes Qbar (as
-// spreading strengths), the target-side x-gradient and the explicit y-term,
-// and per-block partial sums of the bandwidth gradient.
+// Where a moment of the degrees gathered at the samples lies: the F2 fields of
+// the forward pass first (s-fields, then nt per response), then the extra
+// moments (mono_x: the s-fields of degree 2l + 1, then degree l + 1 per
+// response).  all: index in the graded list of every monomial.
+__device__ __forceinline__ int s_slot(int k, int ns, int F2) { return k < ns ? k : F2 + k - ns; }
+__device__ __forceinline__ int t_slot(int k, int r, int ns, int nt, int F2, int nsx, int ntx) {
+  return k < nt ? ns + r * nt + k : F2 + (nsx - ns) + r * (ntx - nt) + k - nt;
+}
+
+// Per-sample adjoints (FP64 plans and 3-D local linear).  V holds the F2 field
+// values and the extra moments.  Writes Qbar (as spreading strengths), the
+// target-side x-gradient and the explicit y-term.
 template <typename T, int D>
 __global__ void __launch_bounds__(kE1Threads)
-adjoint_kernel(MonoTab mono, const BwDev* __restrict__ bwt, int b, int order, int64_t n, int F2,
-               int n_probes, const T* __restrict__ V, const T* __restrict__ str,
-               const double* __restrict__ sums, int nacc, const double* __restrict__ sc,
-               T* __restrict__ qbar, T* __restrict__ dxt, T* __restrict__ dye,
-               double* __restrict__ part) {
-  __shared__ double red[kE1Threads / 32][3];
+adjoint_kernel(MonoTab mono, MonoTab all, const BwDev* __restrict__ bwt, int b, int order,
+               int64_t n, int F2, int n_probes, const T* __restrict__ V,
+               const T* __restrict__ str, const double* __restrict__ sums, int nacc,
+               const double* __restrict__ sc, T* __restrict__ qbar, T* __restrict__ dxt,
+               T* __restrict__ dye) {
   const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   const bool valid = s < n;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const BwDev& B = bwt[b];
   const int ns = mono.n, nt = mono.nt, p = nt;
-  double dth[3] = {0, 0, 0};
   if (valid) {
     const double* sb = sums + int64_t(b) * nacc;
     const double L_rss = sc[0], L_trn = sc[1];
@@ -133,7 +153,29 @@ adjoint_kernel(MonoTab mono, const BwDev* __restrict__ bwt, int b, int order, in
       for (int i = 0; i < p; ++i) a[i] = Sinv[i][0];
     double dx_t[3] = {0, 0, 0};
     const int R = 1 + n_probes;
-    const int nblk = 1 + 2 * D;
+    // the neighbours f + e_d and f - e_d of the monomials
+    int up[kMaxP + 1][3], dn[kMaxP + 1][3];
+    double is2[3] = {0, 0, 0};
+    for (int d = 0; d < D; ++d) {
+      is2[d] = B.isigma[d] * B.isigma[d];
+      for (int k = 0; k < ns; ++k) {
+        const int e0 = all.e[k][0], e1 = all.e[k][1], e2 = all.e[k][2];
+        up[k][d] = mono_index(all, all.n, e0 + (d == 0), e1 + (d == 1), e2 + (d == 2));
+        dn[k][d] = all.e[k][d] > 0
+                       ? mono_index(all, all.n, e0 - (d == 0), e1 - (d == 1), e2 - (d == 2))
+                       : 0;
+      }
+    }
+    auto grad = [&](int k, int d, int r) {  // dQ/dq_d of s-field k (r < 0) or t-field k of r
+      const int u = r < 0 ? s_slot(up[k][d], ns, F2)
+                          : t_slot(up[k][d], r, ns, nt, F2, all.n, all.nt);
+      double v = double(V[int64_t(u) * n + s]) * is2[d];
+      if (all.e[k][d] > 0) {
+        const int l = r < 0 ? dn[k][d] : ns + r * nt + dn[k][d];
+        v -= all.e[k][d] * double(V[int64_t(l) * n + s]);
+      }
+      return v;
+    };
     for (int r = 0; r < R && ok; ++r) {
       double t[kMaxP];
       for (int k = 0; k < p; ++k) t[k] = double(V[int64_t(ns + r * nt + k) * n + s]);
@@ -157,8 +199,7 @@ adjoint_kernel(MonoTab mono, const BwDev* __restrict__ bwt, int b, int order, in
         const int f = ns + r * nt + k;
         const double q = gr * a[k];
         qbar[int64_t(f) * n + s] = T(q);
-        for (int d = 0; d < D; ++d) dx_t[d] += q * double(V[(int64_t(1 + d) * F2 + f) * n + s]);
-        for (int d = 0; d < D; ++d) dth[d] += q * double(V[(int64_t(1 + D + d) * F2 + f) * n + s]);
+        for (int d = 0; d < D; ++d) dx_t[d] += q * grad(k, d, r);
       }
     }
     // s-field adjoints: -sum_(a+b=g) a_a bbar_b over ordered pairs
@@ -172,26 +213,13 @@ adjoint_kernel(MonoTab mono, const BwDev* __restrict__ bwt, int b, int order, in
                 mono.e[i][2] + mono.e[j][2] == mono.e[gf][2])
               q -= a[i] * bbar[j];
       qbar[int64_t(gf) * n + s] = T(q);
-      for (int d = 0; d < D; ++d) dx_t[d] += q * double(V[(int64_t(1 + d) * F2 + gf) * n + s]);
-      for (int d = 0; d < D; ++d) dth[d] += q * double(V[(int64_t(1 + D + d) * F2 + gf) * n + s]);
+      for (int d = 0; d < D; ++d) dx_t[d] += q * grad(gf, d, -1);
     }
     if (!ok) {
       for (int f = 0; f < F2; ++f) qbar[int64_t(f) * n + s] = T(0);
       dye[s] = T(0);
     }
     for (int d = 0; d < D; ++d) dxt[int64_t(d) * n + s] = T(dx_t[d]);
-    (void)nblk;
-  }
-  for (int d = 0; d < 3; ++d) {
-    double v = dth[d];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (lane == 0) red[warp][d] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < 3) {
-    double t = 0.0;
-    for (int wv = 0; wv < kE1Threads / 32; ++wv) t += red[wv][threadIdx.x];
-    part[int64_t(blockIdx.x) * 3 + threadIdx.x] = t;
   }
 }
 
@@ -248,121 +276,144 @@ __device__ __forceinline__ bool sym_inverse_f32(const float (&m)[P][P], float (&
   }
 }
 
-// FP32 form of adjoint_kernel for 1-D / 2-D systems known at compile time
-// (NW: p = 1; local linear: p = D + 1).  Same quantities; FP32 per sample
-// (the FP64 pipe is a small fraction of the FP32 rate on this part), FP64
-// for the block sums of the bandwidth gradient.
+// Neighbours of the monomials at compile time: up[k][d] is the index of
+// e_k + e_d in the graded list of degree <= DEG + 1, dn[k][d] of e_k - e_d, and
+// e[k][d] the exponent.
+template <int D, int DEG>
+struct MonoNb {
+  int n, up[mono_count(D, DEG)][D], dn[mono_count(D, DEG)][D], e[mono_count(D, DEG)][D];
+};
+template <int D, int DEG>
+__host__ __device__ constexpr MonoNb<D, DEG> make_mono_nb() {
+  const MonoChain c = make_mono_chain(D, DEG + 1);
+  int e[kMaxMono][3] = {};
+  for (int f = 1; f < c.n; ++f) {
+    for (int j = 0; j < 3; ++j) e[f][j] = e[c.parent[f]][j];
+    e[f][c.axis[f]] += 1;
+  }
+  MonoNb<D, DEG> t{};
+  t.n = mono_count(D, DEG);
+  for (int k = 0; k < t.n; ++k)
+    for (int d = 0; d < D; ++d) {
+      t.e[k][d] = e[k][d];
+      for (int f = 0; f < c.n; ++f) {
+        bool u = true, l = true;
+        for (int j = 0; j < 3; ++j) {
+          if (e[f][j] != e[k][j] + (j == d ? 1 : 0)) u = false;
+          if (e[f][j] != e[k][j] - (j == d ? 1 : 0)) l = false;
+        }
+        if (u) t.up[k][d] = f;
+        if (l) t.dn[k][d] = f;
+      }
+    }
+  return t;
+}
+
+// FP32 form of adjoint_kernel for systems of at most three unknowns known at
+// compile time (NW: p = 1; local linear: p = D + 1).  Same quantities in FP32 per
+// sample (the FP64 pipe is a small fraction of the FP32 rate on this part).
+// Bound by HBM: 2-D local linear with eleven strengths reads 88 values a
+// sample and writes 42.
 template <int D, int ORD>
 __global__ void __launch_bounds__(kE1Threads)
 adjoint_f32_kernel(const BwDev* __restrict__ bwt, int b, int64_t n, int F2, int n_probes,
                    const float* __restrict__ V, const float* __restrict__ str,
-                   const double* __restrict__ sums, int nacc, const double* __restrict__ sc,
-                   float* __restrict__ qbar, float* __restrict__ dxt, float* __restrict__ dye,
-                   double* __restrict__ part) {
-  constexpr int P = ORD == 0 ? 1 : D + 1;
-  constexpr int NS = ORD == 0 ? 1 : (D + 1) * (D + 2) / 2;
-  __shared__ double red[kE1Threads / 32][3];
+                   const double* __restrict__ sc, float* __restrict__ qbar,
+                   float* __restrict__ dxt, float* __restrict__ dye) {
+  constexpr int P = mono_count(D, ORD), PX = mono_count(D, ORD + 1);
+  constexpr int NS = mono_count(D, 2 * ORD), NSX = mono_count(D, 2 * ORD + 1);
+  constexpr auto snb = make_mono_nb<D, 2 * ORD>();
+  constexpr auto tnb = make_mono_nb<D, ORD>();
   const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  const bool valid = s < n;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (s >= n) return;
   const BwDev& B = bwt[b];
-  float dth[3] = {0.f, 0.f, 0.f};
-  if (valid) {
-    const double* sb = sums + int64_t(b) * nacc;
-    const float L_rss = float(sc[0]), L_trn = float(sc[1]);
-    float dsc[P];
-    dsc[0] = 1.f;
+  const float2* fac = reinterpret_cast<const float2*>(sc + 16);
+  float dsc[P], is2[D];
+  dsc[0] = 1.f;
 #pragma unroll
-    for (int k = 1; k < P; ++k) dsc[k] = float(1.0 / B.sigma[k - 1]);
-    float sv[NS];
+  for (int k = 1; k < P; ++k) dsc[k] = float(B.isigma[k - 1]);
 #pragma unroll
-    for (int k = 0; k < NS; ++k) sv[k] = V[int64_t(k) * n + s];
-    float m[P][P], mi[P][P];
+  for (int d = 0; d < D; ++d) is2[d] = float(B.isigma[d] * B.isigma[d]);
+  float sv[NSX];
 #pragma unroll
-    for (int i = 0; i < P; ++i)
+  for (int k = 0; k < NSX; ++k) sv[k] = V[int64_t(k < NS ? k : F2 + k - NS) * n + s];
+  float m[P][P], mi[P][P];
 #pragma unroll
-      for (int j = 0; j < P; ++j) m[i][j] = sv[sidx<D>(i, j)] * (dsc[i] * dsc[j]);
-    const bool ok = sym_inverse_f32<P>(m, mi);
-    float Sinv[P][P];
+  for (int i = 0; i < P; ++i)
 #pragma unroll
-    for (int i = 0; i < P; ++i)
+    for (int j = 0; j < P; ++j) m[i][j] = sv[sidx<D>(i, j)] * (dsc[i] * dsc[j]);
+  const bool ok = sym_inverse_f32<P>(m, mi);
+  float Sinv[P][P];
 #pragma unroll
-      for (int j = 0; j < P; ++j) Sinv[i][j] = ok ? mi[i][j] * (dsc[i] * dsc[j]) : 0.f;
-    float a[P], bbar[P];
+  for (int i = 0; i < P; ++i)
+#pragma unroll
+    for (int j = 0; j < P; ++j) Sinv[i][j] = ok ? mi[i][j] * (dsc[i] * dsc[j]) : 0.f;
+  float a[P], bbar[P];
+#pragma unroll
+  for (int i = 0; i < P; ++i) {
+    a[i] = Sinv[i][0];
+    bbar[i] = 0.f;
+  }
+  float dx_t[D];
+#pragma unroll
+  for (int d = 0; d < D; ++d) dx_t[d] = 0.f;
+  const int R = 1 + n_probes;
+#pragma unroll 2
+  for (int r = 0; r < R; ++r) {
+    float t[PX];
+#pragma unroll
+    for (int k = 0; k < PX; ++k)
+      t[k] = V[int64_t(k < P ? NS + r * P + k : F2 + (NSX - NS) + r * (PX - P) + k - P) * n + s];
+    float mh = 0.f;
+#pragma unroll
+    for (int k = 0; k < P; ++k) mh += a[k] * t[k];
+    const float c = str[int64_t(1 + r) * n + s];
+    const float2 fr = fac[r];
+    const float v = r == 0 ? c - mh : c;
+    float gr = ok ? fmaf(v, fr.x, v * fr.y) : 0.f;
+    if (r == 0) {
+      dye[s] = gr;
+      gr = -gr;
+    }
 #pragma unroll
     for (int i = 0; i < P; ++i) {
-      a[i] = Sinv[i][0];
-      bbar[i] = 0.f;
+      float beta = 0.f;
+#pragma unroll
+      for (int k = 0; k < P; ++k) beta += Sinv[i][k] * t[k];
+      bbar[i] += gr * beta;
     }
-    float dx_t[3] = {0.f, 0.f, 0.f};
-    const int R = 1 + n_probes;
-#pragma unroll 2
-    for (int r = 0; r < R; ++r) {
-      float t[P];
 #pragma unroll
-      for (int k = 0; k < P; ++k) t[k] = V[int64_t(NS + r * P + k) * n + s];
-      float mh = 0.f;
-#pragma unroll
-      for (int k = 0; k < P; ++k) mh += a[k] * t[k];
-      const float c = str[int64_t(1 + r) * n + s];
-      float gr;
-      if (r == 0) {
-        gr = -2.f * L_rss * (c - mh);
-        dye[s] = ok ? 2.f * L_rss * (c - mh) : 0.f;
-      } else {
-        gr = L_trn * c / float(sb[1 + n_probes + (r - 1)]);
-      }
-      if (!ok) gr = 0.f;
-#pragma unroll
-      for (int i = 0; i < P; ++i) {
-        float beta = 0.f;
-#pragma unroll
-        for (int k = 0; k < P; ++k) beta += Sinv[i][k] * t[k];
-        bbar[i] += gr * beta;
-      }
-#pragma unroll
-      for (int k = 0; k < P; ++k) {
-        const int f = NS + r * P + k;
-        const float q = gr * a[k];
-        qbar[int64_t(f) * n + s] = q;
-#pragma unroll
-        for (int d = 0; d < D; ++d) {
-          dx_t[d] += q * V[(int64_t(1 + d) * F2 + f) * n + s];
-          dth[d] += q * V[(int64_t(1 + D + d) * F2 + f) * n + s];
-        }
-      }
-    }
-    // s-field adjoints: -sum_(a+b=g) a_a bbar_b over ordered pairs
-    float qs[NS];
-#pragma unroll
-    for (int g = 0; g < NS; ++g) qs[g] = 0.f;
-#pragma unroll
-    for (int i = 0; i < P; ++i)
-#pragma unroll
-      for (int j = 0; j < P; ++j) qs[sidx<D>(i, j)] -= a[i] * bbar[j];
-#pragma unroll
-    for (int g = 0; g < NS; ++g) {
-      qbar[int64_t(g) * n + s] = qs[g];
+    for (int k = 0; k < P; ++k) {
+      const float q = gr * a[k];
+      qbar[int64_t(NS + r * P + k) * n + s] = q;
 #pragma unroll
       for (int d = 0; d < D; ++d) {
-        dx_t[d] += qs[g] * V[(int64_t(1 + d) * F2 + g) * n + s];
-        dth[d] += qs[g] * V[(int64_t(1 + D + d) * F2 + g) * n + s];
+        float gd = t[tnb.up[k][d]] * is2[d];
+        if (tnb.e[k][d] > 0) gd -= float(tnb.e[k][d]) * t[tnb.dn[k][d]];
+        dx_t[d] += q * gd;
       }
     }
+  }
+  // s-field adjoints: -sum_(a+b=g) a_a bbar_b over ordered pairs
+  float qs[NS];
 #pragma unroll
-    for (int d = 0; d < D; ++d) dxt[int64_t(d) * n + s] = dx_t[d];
+  for (int g = 0; g < NS; ++g) qs[g] = 0.f;
+#pragma unroll
+  for (int i = 0; i < P; ++i)
+#pragma unroll
+    for (int j = 0; j < P; ++j) qs[sidx<D>(i, j)] -= a[i] * bbar[j];
+#pragma unroll
+  for (int g = 0; g < NS; ++g) {
+    qbar[int64_t(g) * n + s] = qs[g];
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      float gd = sv[snb.up[g][d]] * is2[d];
+      if (snb.e[g][d] > 0) gd -= float(snb.e[g][d]) * sv[snb.dn[g][d]];
+      dx_t[d] += qs[g] * gd;
+    }
   }
-  for (int d = 0; d < 3; ++d) {
-    double v = double(dth[d]);
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (lane == 0) red[warp][d] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < 3) {
-    double t = 0.0;
-    for (int wv = 0; wv < kE1Threads / 32; ++wv) t += red[wv][threadIdx.x];
-    part[int64_t(blockIdx.x) * 3 + threadIdx.x] = t;
-  }
+#pragma unroll
+  for (int d = 0; d < D; ++d) dxt[int64_t(d) * n + s] = dx_t[d];
 }
 
 // Combine: dy_i = adjoint y-field + explicit term; dx_(i,d) = sum over
@@ -407,21 +458,6 @@ __global__ void combine_kernel(int64_t n, int n_probes, const T* __restrict__ Va
   }
 }
 
-__global__ void reduce_theta(const double* __restrict__ part, int64_t nblk, int D,
-                             double* __restrict__ out) {
-  __shared__ double sh[256];
-  const int d = blockIdx.x;
-  double t = 0.0;
-  for (int64_t k = threadIdx.x; k < nblk; k += blockDim.x) t += part[k * 3 + d];
-  sh[threadIdx.x] = t;
-  __syncthreads();
-  for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-    if (threadIdx.x < st) sh[threadIdx.x] += sh[threadIdx.x + st];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) out[d] = sh[0];
-}
-
 }  // namespace
 
 cudaError_t run_loss_scalars(fkreg_plan_s* P, int b, int n_probes, cudaStream_t st) {
@@ -447,8 +483,7 @@ static cudaError_t adjoint_t(fkreg_plan_s* P, int b, int n_probes, cudaStream_t 
 #define FK_F(DD, OO)                                                                            \
   adjoint_f32_kernel<DD, OO><<<blocks, kE1Threads, 0, st>>>(                                    \
       wsp<BwDev>(P, P->r_bw), b, P->n, F2, n_probes, wsp<float>(P, P->r_bV),                   \
-      wsp<float>(P, P->r_str), sums, nacc, wsp<double>(P, P->r_bsc), qbar, dxt, dye,           \
-      wsp<double>(P, P->r_bpart))
+      wsp<float>(P, P->r_str), wsp<double>(P, P->r_bsc), qbar, dxt, dye)
       if (P->order == 0) {
         if (P->d == 1) FK_F(1, 0);
         else if (P->d == 2) FK_F(2, 0);
@@ -464,9 +499,9 @@ static cudaError_t adjoint_t(fkreg_plan_s* P, int b, int n_probes, cudaStream_t 
   }
 #define FK_A(DD)                                                                              \
   adjoint_kernel<T, DD><<<blocks, kE1Threads, 0, st>>>(                                       \
-      P->mono, wsp<BwDev>(P, P->r_bw), b, P->order, P->n, F2, n_probes, wsp<T>(P, P->r_bV),  \
-      wsp<T>(P, P->r_str), sums, nacc, wsp<double>(P, P->r_bsc), qbar, dxt, dye,             \
-      wsp<double>(P, P->r_bpart))
+      P->mono, P->mono_all, wsp<BwDev>(P, P->r_bw), b, P->order, P->n, F2, n_probes,          \
+      wsp<T>(P, P->r_bV), wsp<T>(P, P->r_str), sums, nacc, wsp<double>(P, P->r_bsc), qbar,    \
+      dxt, dye)
   if (P->d == 1)
     FK_A(1);
   else if (P->d == 2)
@@ -484,8 +519,7 @@ cudaError_t run_adjoint(fkreg_plan_s* P, int b, int n_probes, cudaStream_t st) {
 }
 
 template <typename T>
-static cudaError_t combine_t(fkreg_plan_s* P, int n_probes, void* dy, void* dx, double* dlogh,
-                             cudaStream_t st) {
+static cudaError_t combine_t(fkreg_plan_s* P, int n_probes, void* dy, void* dx, cudaStream_t st) {
   if (P->n > 0) {
     const unsigned blocks = unsigned((P->n + 255) / 256);
     const T* dxt = wsp<T>(P, P->r_bdx);
@@ -505,18 +539,12 @@ static cudaError_t combine_t(fkreg_plan_s* P, int n_probes, void* dy, void* dx, 
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  if (dlogh) {
-    const int64_t nblk = (P->n + kE1Threads - 1) / kE1Threads;
-    reduce_theta<<<P->d, 256, 0, st>>>(wsp<double>(P, P->r_bpart), nblk, P->d, dlogh);
-    P->launches += 1;
-  }
   return cudaGetLastError();
 }
 
-cudaError_t run_combine(fkreg_plan_s* P, int n_probes, void* dy, void* dx, double* dlogh,
-                        cudaStream_t st) {
-  return P->prec == FKREG_F32 ? combine_t<float>(P, n_probes, dy, dx, dlogh, st)
-                              : combine_t<double>(P, n_probes, dy, dx, dlogh, st);
+cudaError_t run_combine(fkreg_plan_s* P, int n_probes, void* dy, void* dx, cudaStream_t st) {
+  return P->prec == FKREG_F32 ? combine_t<float>(P, n_probes, dy, dx, st)
+                              : combine_t<double>(P, n_probes, dy, dx, st);
 }
 
 }  // namespace fk

@@ -121,6 +121,7 @@ struct BwDev {
 struct MonoTab {
   int n;               // monomials of degree <= 2l  (s-fields)
   int nt;              // monomials of degree <= l   (t-fields)
+  int toff;            // where the t-monomials start in e (0: a prefix of the s-monomials)
   int e[kMaxMono][kMaxD];
 };
 
@@ -136,6 +137,10 @@ struct fkreg_plan_s {
   fkreg_geometry g{};
   fk::GeoDev geo{};
   fk::MonoTab mono{};
+  // backward: monomials of degree <= 2l + 1 in the graded order (n), and the
+  // ones that the gradients need beyond the plan's fields: s of degree 2l + 1
+  // (n) and t of degree l + 1 (nt, from toff)
+  fk::MonoTab mono_all{}, mono_x{};
   fk::PhiPoly poly{};           // FP64 plans
   int64_t max_n = 0;
   int d = 0, order = 0, prec = 0, ns = 0, nt = 0, p = 0;
@@ -158,10 +163,11 @@ struct fkreg_plan_s {
       r_binstart, r_nsub, r_substart, r_subbin, r_subfirst, r_hist, r_hist2, r_dtot, r_scan, r_str,
       r_fine, r_spec, r_gspec, r_gfield, r_t2spec, r_t2field, r_part, r_smax, r_fftwork,
       r_fftwork_g,
-      r_bV, r_bdx, r_bsc, r_bpart, r_gmask, r_gadj, r_gpart, r_gavec;
+      r_bV, r_bdx, r_bsc, r_gmask, r_gadj, r_gpart, r_gavec;
   bool backward = false;        // workspace reserved for fkreg_backward
   bool direct = false;          // compact kernel: direct sums instead of the NUFFT
   int f2bwd = 0;                // fields of the backward passes (one response + probes)
+  int fxbwd = 0;                // extra moment fields of the backward (mono_x)
   size_t ws_bytes = 0;
   size_t fft_work_reserved = 0;
   size_t fft_work_reserved_g = 0;  // inverse grid transforms (their own area: they overlap)
@@ -227,10 +233,12 @@ cudaError_t run_logres_strengths(fkreg_plan_s* P, const void* y, const void* mha
 // spectral.cu
 cudaError_t run_kmul_grid(fkreg_plan_s* P, int str_dens, int str_rhs, int nrhs_fields,
                           int bw_first, int bw_count, void* out_spec, cudaStream_t s);
-cudaError_t run_kmul_t2(fkreg_plan_s* P, int b, int str_dens, int str_rhs, int n_rhs_str,
-                        cudaStream_t s);
-cudaError_t run_kmul_t2_mode(fkreg_plan_s* P, int b, int str_dens, int str_rhs, int n_rhs_str,
-                             int kind, int axis, cudaStream_t s);
+cudaError_t run_kmul_t2(fkreg_plan_s* P, int b, const MonoTab& mono, int str_dens, int str_rhs,
+                        int n_rhs_str, cudaStream_t s);
+// d GCV / d log sigma from the spectra of the strengths and of the spread
+// adjoints (strength slots sb ..), with run_dlogh_lattice_blocks x 3 partial sums
+cudaError_t run_dlogh_spread(fkreg_plan_s* P, int b, int n_rhs_str, int sb, double* part,
+                             double* dlogh, cudaStream_t s);
 cudaError_t run_kmul_adj(fkreg_plan_s* P, int b, int sb, int n_classes, cudaStream_t s);
 // grid-estimate backward: type-2 spectra of the adjoint functions of the
 // lattice adjoint fields (their R2C spectra E [fgrid][L half]), and
@@ -251,11 +259,11 @@ cudaError_t run_combine_grid(fkreg_plan_s* P, int nrhs, const void* V, void* dy,
 // backward.cu
 cudaError_t run_gather_fields(fkreg_plan_s* P, int b, int F, void* V, cudaStream_t s);
 // Persistent interpolation kernel (FP32, width 7, 1-D / 2-D, F2 <= 64):
-// launched only when it applies (*launched); vout != NULL selects the
-// gather-only form (F2 fields into vout[f][n]).
+// launched only when it applies (*launched); vout != NULL takes the F2 fields
+// (vout[f][n]), which is all that the gather-only form (gonly) does.
 cudaError_t run_interp_direct(fkreg_plan_s* P, int b, int n_rhs_real, int n_probes,
                               void* mhat_at_x, cudaStream_t st, int nacc, int F2, void* vout,
-                              bool* launched);
+                              bool gonly, bool* launched);
 // Lane-per-sample kernels of interp_lane.cuh (compile-time widths, every
 // dimension and order), launched only when they apply (*launched).
 cudaError_t run_interp_lane_f32(fkreg_plan_s* P, int b, int n_rhs_real, int n_probes,
@@ -271,8 +279,7 @@ cudaError_t run_interp_global_lane(fkreg_plan_s* P, int b, int n_rhs_real, int n
                                    void* vout, bool* launched);
 cudaError_t run_loss_scalars(fkreg_plan_s* P, int b, int n_probes, cudaStream_t s);
 cudaError_t run_adjoint(fkreg_plan_s* P, int b, int n_probes, cudaStream_t s);
-cudaError_t run_combine(fkreg_plan_s* P, int n_probes, void* dy, void* dx, double* dlogh,
-                        cudaStream_t s);
+cudaError_t run_combine(fkreg_plan_s* P, int n_probes, void* dy, void* dx, cudaStream_t s);
 
 // solve.cu
 // avec (may be null): [bw][p][M] the solved weights a_k / tscale_k of each
@@ -282,8 +289,9 @@ cudaError_t run_grid_solve(fkreg_plan_s* P, int bw_first, int bw_count, int nrhs
 // sigma2[b][r][M] = sum_k avec[b][k] t_(r,k) from the grid t-fields alone
 // (r_gfield holds nrhs_fields x p t-fields; no s-fields, no solve)
 cudaError_t run_grid_apply(fkreg_plan_s* P, int b, int nrhs_fields, void* sigma2, cudaStream_t s);
-cudaError_t run_interp(fkreg_plan_s* P, int b, int n_rhs_str, int n_probes, const void* y,
-                       void* mhat_at_x, cudaStream_t s);
+// keep (may be null): also the fields themselves, [ns + (n_rhs_str + n_probes) nt][n]
+cudaError_t run_interp(fkreg_plan_s* P, int b, int n_rhs_str, int n_probes, void* mhat_at_x,
+                       void* keep, cudaStream_t s);
 // direct path (compact kernels): grid fields of strengths [str_first, str_first + nstr)
 // plus the s-fields, bandwidths [bw_first, bw_first + bw_count), into r_gfield
 cudaError_t run_direct_grid(fkreg_plan_s* P, int str_first, int nstr, int bw_first,

@@ -221,7 +221,7 @@ cudaError_t launch_interp_w(fkreg_plan_s* P, int b, int n_rhs_real, int n_probes
 
 template <typename T>
 cudaError_t launch_interp(fkreg_plan_s* P, int b, int n_rhs_str, int n_probes, void* mhat_at_x,
-                          cudaStream_t st) {
+                          void* keep, bool* kept, cudaStream_t st) {
   const int n_rhs_real = n_rhs_str;
   const int nacc = n_rhs_real + 2 * n_probes + 1;
   if (nacc > kMaxAcc) return cudaErrorInvalidValue;
@@ -230,7 +230,8 @@ cudaError_t launch_interp(fkreg_plan_s* P, int b, int n_rhs_str, int n_probes, v
   if (sizeof(T) == 4) {
     bool used = false;
     cudaError_t e =
-        run_interp_direct(P, b, n_rhs_real, n_probes, mhat_at_x, st, nacc, F2, nullptr, &used);
+        run_interp_direct(P, b, n_rhs_real, n_probes, mhat_at_x, st, nacc, F2, keep, false, &used);
+    *kept = used && keep;
     if (used || e != cudaSuccess) return e;
     e = run_interp_global_lane(P, b, n_rhs_real, n_probes, mhat_at_x, st, nacc, F2, nullptr, &used);
     if (used || e != cudaSuccess) return e;
@@ -263,7 +264,7 @@ cudaError_t launch_gather(fkreg_plan_s* P, int b, int F, T* V, cudaStream_t st) 
   if (P->d * P->geo.w > 64 || P->geo.w > kMaxWRun) return cudaErrorInvalidValue;
   if (sizeof(T) == 4) {
     bool used = false;
-    cudaError_t e = run_interp_direct(P, b, 0, 0, nullptr, st, 0, F, V, &used);
+    cudaError_t e = run_interp_direct(P, b, 0, 0, nullptr, st, 0, F, V, true, &used);
     if (used || e != cudaSuccess) return e;
     e = run_interp_global_lane(P, b, 0, 0, nullptr, st, 0, F, V, &used);
     if (used || e != cudaSuccess) return e;
@@ -292,11 +293,17 @@ cudaError_t run_gather_fields(fkreg_plan_s* P, int b, int F, void* V, cudaStream
                               : launch_gather<double>(P, b, F, static_cast<double*>(V), st);
 }
 
-cudaError_t run_interp(fkreg_plan_s* P, int b, int n_rhs_str, int n_probes, const void*,
-                       void* mhat_at_x, cudaStream_t st) {
+cudaError_t run_interp(fkreg_plan_s* P, int b, int n_rhs_str, int n_probes, void* mhat_at_x,
+                       void* keep, cudaStream_t st) {
   if (P->direct) return run_direct_interp(P, b, n_rhs_str, n_probes, mhat_at_x, st);
-  return P->prec == FKREG_F32 ? launch_interp<float>(P, b, n_rhs_str, n_probes, mhat_at_x, st)
-                              : launch_interp<double>(P, b, n_rhs_str, n_probes, mhat_at_x, st);
+  bool kept = false;
+  const cudaError_t e =
+      P->prec == FKREG_F32
+          ? launch_interp<float>(P, b, n_rhs_str, n_probes, mhat_at_x, keep, &kept, st)
+          : launch_interp<double>(P, b, n_rhs_str, n_probes, mhat_at_x, keep, &kept, st);
+  if (e != cudaSuccess || !keep || kept) return e;
+  // kernels that don't store the fields on the way: gather them from the same grid
+  return run_gather_fields(P, b, P->ns + (n_rhs_str + n_probes) * P->nt, keep, st);
 }
 
 // Sum the partials of the last interpolation passes and derive DF and GCV.

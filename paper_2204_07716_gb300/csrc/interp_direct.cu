@@ -9,7 +9,7 @@
 // on the tensor cores (mma_union_gather: split-TF32 products over the
 // union); other warps, and 1-D plans, gather lane per sample with packed FP32
 // FMAs.  The gather-only form (GONLY) writes V[f][s] for the backward instead
-// of phase B.
+// of phase B; the full form writes V beside phase B when it is given one.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -234,7 +234,7 @@ interp_direct_kernel(GeoDev g, const BwDev* __restrict__ bwt, int b, int64_t n,
                                          acc);
         }
       }
-      if (GONLY) {
+      if (GONLY || vout) {
         if (valid)
 #pragma unroll
           for (int q = 0; q < NQ; ++q)
@@ -243,7 +243,7 @@ interp_direct_kernel(GeoDev g, const BwDev* __restrict__ bwt, int b, int64_t n,
               const int f = 4 * q + cc;
               if (f < F2) vout[int64_t(f) * n + s] = quad_comp(acc[q], cc);
             }
-        continue;
+        if (GONLY) continue;
       }
       // phase B: the system of eq. 3 at x_i from the s-fields in registers
       float a[kMaxP] = {0.f, 0.f, 0.f, 0.f};
@@ -401,11 +401,11 @@ cudaError_t launch_direct_q(fkreg_plan_s* P, int b, int n_rhs_real, int n_probes
 // F2 <= 64, two windows fit shared memory); *launched says whether it ran.
 cudaError_t run_interp_direct(fkreg_plan_s* P, int b, int n_rhs_real, int n_probes,
                               void* mhat_at_x, cudaStream_t st, int nacc, int F2, void* vout,
-                              bool* launched) {
+                              bool gonly, bool* launched) {
   *launched = false;
   const int D = P->d;
   if (P->prec != FKREG_F32 || P->geo.w != 7 || D > 2 || F2 > 64 || P->n == 0) return cudaSuccess;
-  if (!vout && P->order > 1) return cudaSuccess;
+  if (!gonly && P->order > 1) return cudaSuccess;
   const BwDev& B = P->bw[b];
   const int rec = t2_record_stride(F2, sizeof(float));
   const int wm0 = tma_window(P->geo, B, 0);
@@ -438,7 +438,7 @@ cudaError_t run_interp_direct(fkreg_plan_s* P, int b, int n_rhs_real, int n_prob
 #define FK_A(DD, OO, GG)                                                                        \
   return launch_direct_q<DD, OO, GG>(P, b, n_rhs_real, n_probes, mhat_at_x, st, nacc, F2, vo,  \
                                      rec, wm0, wm1, pitch, slack, win_floats, nw, smem, grid)
-  if (vout) {
+  if (gonly) {
     if (D == 1) FK_A(1, 0, true);
     FK_A(2, 0, true);
   }

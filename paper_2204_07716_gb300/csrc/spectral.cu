@@ -336,7 +336,8 @@ __global__ void kmul_t2_kernel(GeoDev g, const BwDev* __restrict__ bwt, int b,
     base.x *= sc;
     base.y *= sc;
     for (int f = 0; f < nfld; ++f)
-      out[int64_t(fbase + f) * t2half + j] = mult_field<T, C>(base, m, B, mono, f);
+      out[int64_t(fbase + f) * t2half + j] =
+          mult_field<T, C>(base, m, B, mono, q == 0 ? f : mono.toff + f);
   }
 }
 
@@ -376,8 +377,8 @@ cudaError_t launch_grid(fkreg_plan_s* P, int str_dens, int str_rhs, int nrhs_fie
 }
 
 template <typename T>
-cudaError_t launch_t2(fkreg_plan_s* P, int b, int str_dens, int str_rhs, int n_rhs_str,
-                      cudaStream_t st) {
+cudaError_t launch_t2(fkreg_plan_s* P, int b, const MonoTab& mono, int str_dens, int str_rhs,
+                      int n_rhs_str, cudaStream_t st) {
   using C = typename Cx<T>::type;
   const GeoDev& g = P->geo;
   const int D = P->d;
@@ -394,7 +395,7 @@ cudaError_t launch_t2(fkreg_plan_s* P, int b, int str_dens, int str_rhs, int n_r
   C* o = wsp<C>(P, P->r_t2spec);
 #define FK_KT(DD)                                                                               \
   kmul_t2_kernel<T, DD><<<blocks, 256, 0, st>>>(g, bwt, b, tab, P->phi1_off[0], P->phi1_off[1], \
-                                                P->phi1_off[2], P->mono, F, fhalf, str_dens,    \
+                                                P->phi1_off[2], mono, F, fhalf, str_dens,       \
                                                 str_rhs, n_rhs_str, t2half, o)
   if (D == 1)
     FK_KT(1);
@@ -410,8 +411,6 @@ cudaError_t launch_t2(fkreg_plan_s* P, int b, int str_dens, int str_rhs, int n_r
 
 // ---- multipliers for the backward pass ----------------------------------------
 // Fourier multiplier of field f (monomial exponent e_f) at xi = k / P:
-//  kind 0: conj(w^_f(xi))             forward field T_f(q) = sum_i c_i w_f(x_i - q)
-//  kind 1: 2 pi i xi_d conj(w^_f)     its gradient in the evaluation point q_d
 //  kind 2: d conj(w^_f) / d log sigma_j   (H = diag(sigma^2))
 //  kind 3: w^_f(xi)                   adjoint field sum_m e_m w_f(q - x_m)
 //  kind 4: 2 pi i xi_d w^_f(xi)       adjoint field of the kernel derivative
@@ -448,76 +447,19 @@ __device__ __forceinline__ C field_mult(const MonoTab& mono, int f, int kind, in
     }
     return W;
   }
-  const bool adjoint = kind >= 3;
   if (deg == 0) {
     W.x = m.G;
   } else if (deg == 1) {
-    W.y = (adjoint ? -twopi : twopi) * m.hx[a] * m.G;
+    W.y = -twopi * m.hx[a] * m.G;
   } else {
     W.x = (T(B.H[a * 3 + b]) - fpi2 * m.hx[a] * m.hx[b]) * m.G;
   }
-  if (kind == 1 || kind == 4) {  // times 2 pi i xi_d
+  if (kind == 4) {  // times 2 pi i xi_d
     const T s = twopi * xi[axis];
     const C r{-W.y * s, W.x * s};
     return r;
   }
   return W;
-}
-
-// Type-2 spectra of the forward fields under multiplier `kind` (0, 1, 2), for
-// one bandwidth: thread per (fine half-spectrum index, strength q).
-template <typename T, int D>
-__global__ void kmul_t2_mode_kernel(GeoDev g, const BwDev* __restrict__ bwt, int b,
-                                    const double* __restrict__ tab, int64_t phi1_0, int64_t phi1_1,
-                                    int64_t phi1_2, MonoTab mono,
-                                    const typename Cx<T>::type* __restrict__ F, int64_t fine_half,
-                                    int str_dens, int str_rhs, int n_rhs_str, int kind, int axis,
-                                    int64_t t2half, typename Cx<T>::type* __restrict__ out) {
-  using C = typename Cx<T>::type;
-  const int nq = 1 + n_rhs_str;
-  const int64_t gid = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (gid >= t2half * nq) return;
-  const int64_t j = gid % t2half;
-  const int q = int(gid / t2half);
-  const BwDev& B = bwt[b];
-  const bool dens = q == 0;
-  const int strength = dens ? str_dens : str_rhs + q - 1;
-  const int nfld = dens ? mono.n : mono.nt;
-  const int fbase = dens ? 0 : mono.n + (q - 1) * mono.nt;
-  int64_t kk[3] = {0, 0, 0};
-  bool inside = true;
-  {
-    int64_t rem = j;
-    for (int a = D - 1; a >= 0; --a) {
-      const int64_t nn = (a == D - 1) ? (B.nf[a] / 2 + 1) : B.nf[a];
-      int64_t idx = rem % nn;
-      rem /= nn;
-      int64_t k = (a == D - 1) ? idx : (idx < (B.nf[a] + 1) / 2 ? idx : idx - B.nf[a]);
-      kk[a] = k;
-      if ((k < 0 ? -k : k) > B.K[a] / 2 - 1) inside = false;
-    }
-  }
-  C res[kMaxMono];
-  for (int f = 0; f < kMaxMono; ++f) res[f] = C{T(0), T(0)};
-  if (inside) {
-    const int64_t phi1[3] = {phi1_0, phi1_1, phi1_2};
-    T dec = T(1);
-    T xi[3] = {T(0), T(0), T(0)};
-    for (int a = 0; a < D; ++a) {
-      const int64_t ak = kk[a] < 0 ? -kk[a] : kk[a];
-      dec *= T(tab[phi1[a] + ak] * tab[B.phi2_off[a] + ak] / g.P[a]);
-      xi[a] = T(kk[a]) / T(g.P[a]);
-    }
-    const ModeMul<T> m = mode_mul<T>(g, B, kk, D);
-    C base = fetch_F<T, C>(g, F + int64_t(strength) * fine_half, kk, D);
-    base.x *= dec;
-    base.y *= dec;
-    for (int f = 0; f < nfld; ++f) {
-      const C W = field_mult<T, C>(mono, dens ? f : f, kind, axis, xi, m, B);
-      res[f] = cmul<C, T>(W, base);
-    }
-  }
-  for (int f = 0; f < nfld; ++f) out[int64_t(fbase + f) * t2half + j] = res[f];
 }
 
 // Adjoint fields on bandwidth b's type-2 grid from the spectra E_f of the
@@ -751,6 +693,80 @@ __global__ void dlogh_lattice_kernel(GeoDev g, const BwDev* __restrict__ bwt, in
   }
 }
 
+// d GCV / d log sigma_j of the GCV backward.  The field values at the samples
+// are Q_f(x_i) = sum_k (W_f F_k / prod P) exp(2 pi i k (x_i - lo) / P), so with the
+// spectra E_f[k] = sum_i Qbar_(i,f) exp(-2 pi i k (x_i - lo) / P) of the spread
+// adjoints
+//   sum_i Qbar_(i,f) dQ_f(x_i)/dlog sigma_j = sum_k Re[dW_f/dlog sigma_j (F_k / prod P) conj(E_f[k])]
+// and no derivative field has to be gathered at the samples (two sets of 39
+// fields, 0.7 ms of 4.9 for 2 10^6 samples).  Thread per mode of the half box
+// k_last >= 0 (weight 2 off k_last = 0), the fields summed in the plan's
+// precision, FP64 partial sums part[block][3].
+template <typename T, int D>
+__global__ void dlogh_spread_kernel(GeoDev g, const BwDev* __restrict__ bwt, int b,
+                                    const double* __restrict__ tab, int64_t phi1_0, int64_t phi1_1,
+                                    int64_t phi1_2, MonoTab mono,
+                                    const typename Cx<T>::type* __restrict__ F, int64_t fine_half,
+                                    int n_rhs_str, int sb, int64_t nmodes,
+                                    double* __restrict__ part) {
+  using C = typename Cx<T>::type;
+  __shared__ double red[8][3];
+  const int64_t gid = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  const BwDev& B = bwt[b];
+  double dth[3] = {0.0, 0.0, 0.0};
+  if (gid < nmodes) {
+    int64_t kk[3] = {0, 0, 0};
+    int64_t rem = gid;
+    for (int a = D - 1; a >= 0; --a) {
+      const int64_t hk = B.K[a] / 2 - 1;
+      const int64_t nn = (a == D - 1) ? (hk + 1) : (2 * hk + 1);
+      const int64_t idx = rem % nn;
+      rem /= nn;
+      kk[a] = (a == D - 1) ? idx : idx - hk;
+    }
+    const int64_t phi1[3] = {phi1_0, phi1_1, phi1_2};
+    double dec = 1.0;  // both spectra carry the spreading kernel
+    T xi[3] = {T(0), T(0), T(0)};
+    int64_t fidx = 0;
+    for (int a = 0; a < D; ++a) {
+      const double ip = tab[phi1[a] + (kk[a] < 0 ? -kk[a] : kk[a])];
+      dec *= ip * ip / g.P[a];
+      xi[a] = T(kk[a]) / T(g.P[a]);
+      const int64_t nn = (a == D - 1) ? (g.nf[a] / 2 + 1) : g.nf[a];
+      fidx = fidx * nn + (kk[a] < 0 ? kk[a] + g.nf[a] : kk[a]);
+    }
+    const ModeMul<T> m = mode_mul<T>(g, B, kk, D);
+    T acc[D];
+    for (int j = 0; j < D; ++j) acc[j] = T(0);
+    for (int c = 0; c <= n_rhs_str; ++c) {
+      const C Fk = F[int64_t(c) * fine_half + fidx];
+      const int f0 = c == 0 ? 0 : mono.n + (c - 1) * mono.nt, nf = c == 0 ? mono.n : mono.nt;
+      for (int f = 0; f < nf; ++f) {
+        const C e = F[int64_t(sb + f0 + f) * fine_half + fidx];
+        const T px = Fk.x * e.x + Fk.y * e.y, py = Fk.y * e.x - Fk.x * e.y;
+        for (int j = 0; j < D; ++j) {
+          const C W2 = field_mult<T, C>(mono, f, 2, j, xi, m, B);
+          acc[j] += W2.x * px - W2.y * py;
+        }
+      }
+    }
+    const double wgt = (kk[D - 1] == 0 ? 1.0 : 2.0) * dec;
+    for (int j = 0; j < D; ++j) dth[j] = wgt * double(acc[j]);
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int d = 0; d < 3; ++d) {
+    double v = dth[d];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (lane == 0) red[warp][d] = v;
+  }
+  __syncthreads();
+  if (threadIdx.x < 3) {
+    double t = 0.0;
+    for (int wv = 0; wv < int(blockDim.x >> 5); ++wv) t += red[wv][threadIdx.x];
+    part[int64_t(blockIdx.x) * 3 + threadIdx.x] = t;
+  }
+}
+
 __global__ void sum_partials3(const double* __restrict__ part, int64_t nblk, int D,
                               double* __restrict__ out) {
   __shared__ double sh[256];
@@ -839,35 +855,30 @@ cudaError_t launch_dlogh_lattice(fkreg_plan_s* P, int b, int nrhs, const void* E
 }
 
 template <typename T>
-cudaError_t launch_t2_mode(fkreg_plan_s* P, int b, int str_dens, int str_rhs, int n_rhs_str,
-                           int kind, int axis, cudaStream_t st) {
+cudaError_t launch_dlogh_spread(fkreg_plan_s* P, int b, int n_rhs_str, int sb, double* part,
+                                double* dlogh, cudaStream_t st) {
   using C = typename Cx<T>::type;
   const GeoDev& g = P->geo;
   const int D = P->d;
-  const BwDev& B = P->bw[b];
-  int64_t t2half = 1, fhalf = 1;
-  for (int a = 0; a < D; ++a) {
-    t2half *= (a == D - 1) ? (B.nf[a] / 2 + 1) : B.nf[a];
-    fhalf *= (a == D - 1) ? (g.nf[a] / 2 + 1) : g.nf[a];
-  }
-  const int64_t total = t2half * (1 + n_rhs_str);
-  const unsigned blocks = unsigned((total + 255) / 256);
-  auto* F = wsp<C>(P, P->r_spec);
-  auto* bwt = wsp<BwDev>(P, P->r_bw);
-  auto* tab = wsp<double>(P, P->r_tab);
-  C* o = wsp<C>(P, P->r_t2spec);
-#define FK_KM(DD)                                                                                    \
-  kmul_t2_mode_kernel<T, DD><<<blocks, 256, 0, st>>>(g, bwt, b, tab, P->phi1_off[0], P->phi1_off[1], \
-                                                     P->phi1_off[2], P->mono, F, fhalf, str_dens,    \
-                                                     str_rhs, n_rhs_str, kind, axis, t2half, o)
+  int64_t fhalf = 1;
+  for (int a = 0; a < D; ++a) fhalf *= (a == D - 1) ? (g.nf[a] / 2 + 1) : g.nf[a];
+  const int64_t nmodes = dlogh_modes(P, b);
+  const int64_t nblk = (nmodes + 255) / 256;
+#define FK_DS(DD)                                                                                  \
+  dlogh_spread_kernel<T, DD><<<unsigned(nblk), 256, 0, st>>>(                                      \
+      g, wsp<BwDev>(P, P->r_bw), b, wsp<double>(P, P->r_tab), P->phi1_off[0], P->phi1_off[1],      \
+      P->phi1_off[2], P->mono, wsp<C>(P, P->r_spec), fhalf, n_rhs_str, sb, nmodes, part)
   if (D == 1)
-    FK_KM(1);
+    FK_DS(1);
   else if (D == 2)
-    FK_KM(2);
+    FK_DS(2);
   else
-    FK_KM(3);
-#undef FK_KM
-  P->launches += 1;
+    FK_DS(3);
+#undef FK_DS
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  sum_partials3<<<D, 256, 0, st>>>(part, nblk, D, dlogh);
+  P->launches += 2;
   return cudaGetLastError();
 }
 
@@ -913,22 +924,21 @@ cudaError_t run_kmul_grid(fkreg_plan_s* P, int str_dens, int str_rhs, int nrhs_f
              : launch_grid<double>(P, str_dens, str_rhs, nrhs_fields, bw_first, bw_count, out_spec, st);
 }
 
-cudaError_t run_kmul_t2(fkreg_plan_s* P, int b, int str_dens, int str_rhs, int n_rhs_str,
-                        cudaStream_t st) {
-  return P->prec == FKREG_F32 ? launch_t2<float>(P, b, str_dens, str_rhs, n_rhs_str, st)
-                              : launch_t2<double>(P, b, str_dens, str_rhs, n_rhs_str, st);
-}
-
-cudaError_t run_kmul_t2_mode(fkreg_plan_s* P, int b, int str_dens, int str_rhs, int n_rhs_str,
-                             int kind, int axis, cudaStream_t st) {
-  return P->prec == FKREG_F32
-             ? launch_t2_mode<float>(P, b, str_dens, str_rhs, n_rhs_str, kind, axis, st)
-             : launch_t2_mode<double>(P, b, str_dens, str_rhs, n_rhs_str, kind, axis, st);
+cudaError_t run_kmul_t2(fkreg_plan_s* P, int b, const MonoTab& mono, int str_dens, int str_rhs,
+                        int n_rhs_str, cudaStream_t st) {
+  return P->prec == FKREG_F32 ? launch_t2<float>(P, b, mono, str_dens, str_rhs, n_rhs_str, st)
+                              : launch_t2<double>(P, b, mono, str_dens, str_rhs, n_rhs_str, st);
 }
 
 cudaError_t run_kmul_adj(fkreg_plan_s* P, int b, int sb, int n_classes, cudaStream_t st) {
   return P->prec == FKREG_F32 ? launch_adj<float>(P, b, sb, n_classes, st)
                               : launch_adj<double>(P, b, sb, n_classes, st);
+}
+
+cudaError_t run_dlogh_spread(fkreg_plan_s* P, int b, int n_rhs_str, int sb, double* part,
+                             double* dlogh, cudaStream_t st) {
+  return P->prec == FKREG_F32 ? launch_dlogh_spread<float>(P, b, n_rhs_str, sb, part, dlogh, st)
+                              : launch_dlogh_spread<double>(P, b, n_rhs_str, sb, part, dlogh, st);
 }
 
 cudaError_t run_kmul_adj_lattice(fkreg_plan_s* P, int b, int nrhs, const void* E, cudaStream_t st) {
