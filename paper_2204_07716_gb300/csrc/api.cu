@@ -131,6 +131,7 @@ namespace fk {
 // outputs exec_fft then interleaves into cell records, kind 3: forward R2C
 // (the lattice adjoint fields of the grid-estimate backward)
 fkreg_status fft_get(fkreg_plan_s* P, int kind, const int64_t* dims, int batch, cufftHandle* h) {
+  if (fft1d_applies(P, dims[0])) return FKREG_OK;  // no library plan is needed
   auto key = std::make_tuple(kind, dims[0], P->d > 1 ? dims[1] : 1, P->d > 2 ? dims[2] : 1, batch);
   auto it = P->ffts.find(key);
   if (it != P->ffts.end()) {
@@ -316,6 +317,14 @@ fkreg_status fkreg_plan_create(const fkreg_opts* opts, int64_t max_n, fkreg_plan
   L.take(P->r_err, 256);
   L.take(P->r_bw, sizeof(fk::BwDev) * P->nbw);
   L.take(P->r_tab, sizeof(double) * std::max<size_t>(1, P->tab.size()));
+  // 1-D transforms of up to 4096 points are the library's own (fft1d.cu)
+  if (!P->direct && d == 1) {
+    std::vector<int64_t> lens = {P->g.nf[0], P->g.ldft[0]};
+    for (const auto& B : P->bw) lens.push_back(B.nf[0]);
+    for (int64_t n : lens)
+      if (fk::fft1d_applies(P, n)) fk::fft1d_add_roots(P, n);
+  }
+  L.take(P->r_roots, T * std::max<size_t>(2, P->root_tab.size()));
   L.take(P->r_xs, T * d * std::max<int64_t>(1, max_n));
   for (Region* r : {&P->r_keys0, &P->r_vals0, &P->r_keys1, &P->r_vals1})
     L.take(*r, 4 * std::max<int64_t>(1, max_n));
@@ -460,6 +469,17 @@ fkreg_status fkreg_set_workspace(fkreg_plan P, void* ws, size_t bytes, void* str
       (e = cudaMemcpyAsync(P->ws + P->r_tab.off, P->tab.data(), sizeof(double) * P->tab.size(),
                            cudaMemcpyHostToDevice, s)) != cudaSuccess)
     return cuda_err(P, e, "upload tables");
+  std::vector<float> roots_f;
+  if (!P->root_tab.empty()) {
+    const void* src = P->root_tab.data();
+    if (P->prec == FKREG_F32) {
+      roots_f.assign(P->root_tab.begin(), P->root_tab.end());
+      src = roots_f.data();
+    }
+    if ((e = cudaMemcpyAsync(P->ws + P->r_roots.off, src, P->tsize * P->root_tab.size(),
+                             cudaMemcpyHostToDevice, s)) != cudaSuccess)
+      return cuda_err(P, e, "upload roots of unity");
+  }
   // the host tables must outlive the copies: wait for them
   if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_err(P, e, "sync");
   P->points_set = false;
@@ -511,6 +531,14 @@ namespace {
 fkreg_status exec_fft(fkreg_plan_s* P, int kind, const int64_t* dims, int batch, void* in, void* out,
                       cudaStream_t s) {
   const bool fwd = kind == 0 || kind == 3;
+  if (fk::fft1d_applies(P, dims[0])) {
+    const int64_t rec = fk::t2_record_stride(batch, P->tsize);
+    const cudaError_t e =
+        fwd ? fk::run_fft1d_r2c(P, dims[0], batch, in, out, s)
+            : (kind == 2 ? fk::run_fft1d_c2r(P, dims[0], batch, in, out, 1, rec, s)  // cell records
+                         : fk::run_fft1d_c2r(P, dims[0], batch, in, out, dims[0], 1, s));
+    return e == cudaSuccess ? FKREG_OK : cuda_err(P, e, "1-D transform");
+  }
   cufftHandle h;
   fkreg_status st = fk::fft_get(P, kind, dims, batch, &h);
   if (st != FKREG_OK) return st;

@@ -152,6 +152,8 @@ struct fkreg_plan_s {
   std::vector<fk::BwDev> bw;    // host copy of the bandwidth table
   std::vector<double> tab;      // 1/phihat tables (type-1 per axis, then type-2)
   int64_t phi1_off[3] = {0, 0, 0};
+  std::map<int64_t, int64_t> roots;  // 1-D transform lengths -> first root (complex) in root_tab
+  std::vector<double> root_tab;      // roots of unity (re, im)
   int64_t nbins_total = 0;
   int64_t nsub_max = 0;
   int64_t nblk_interp = 0;      // blocks of the interpolation kernel (partials)
@@ -159,7 +161,7 @@ struct fkreg_plan_s {
   int nacc = 0;                 // accumulators per (block, bandwidth)
 
   // workspace regions
-  fk::Region r_err, r_bw, r_tab, r_xs, r_keys0, r_vals0, r_keys1, r_vals1, r_counts,
+  fk::Region r_err, r_bw, r_tab, r_roots, r_xs, r_keys0, r_vals0, r_keys1, r_vals1, r_counts,
       r_binstart, r_nsub, r_substart, r_subbin, r_subfirst, r_hist, r_hist2, r_dtot, r_scan, r_str,
       r_fine, r_spec, r_gspec, r_gfield, r_t2spec, r_t2field, r_part, r_smax, r_fftwork,
       r_fftwork_g,
@@ -312,6 +314,15 @@ int t2_record_stride(int F2, size_t tsize);
 // [cell][t2_record_stride(F, tsize)] at dst.
 cudaError_t run_t2_interleave(fkreg_plan_s* P, const int64_t* dims, int F, const void* src,
                               void* dst, cudaStream_t st);
+
+// fft1d.cu: transforms of 1-D plans in one launch; a real row of n, spectra of n/2 + 1
+bool fft1d_applies(const fkreg_plan_s* P, int64_t n);
+void fft1d_add_roots(fkreg_plan_s* P, int64_t n);
+cudaError_t run_fft1d_r2c(fkreg_plan_s* P, int64_t n, int batch, const void* in, void* out,
+                          cudaStream_t s);
+// value i of row k goes to out[k * row + i * elem]
+cudaError_t run_fft1d_c2r(fkreg_plan_s* P, int64_t n, int batch, const void* in, void* out,
+                          int64_t row, int64_t elem, cudaStream_t s);
 
 // fft helpers (api.cu)
 fkreg_status fft_get(fkreg_plan_s* P, int kind, const int64_t* dims, int batch, cufftHandle* h);
