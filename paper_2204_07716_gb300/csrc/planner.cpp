@@ -149,21 +149,45 @@ void spread_phi_poly(int kind, int w, double beta, PhiPoly* out) {
 }
 
 
-void spread_phihat(int kind, int w, double beta, int64_t nf, int64_t nk, double* out) {
-  // phi is even: phihat(k) = 2 * integral_0^{w/2} phi(z) cos(2 pi k z / nf) dz.
-  // The ES kernel has a square-root edge, so use many nodes.
-  const int q = 8 * w + 64;
-  std::vector<double> x, wt;
-  gauss_legendre(q, &x, &wt);
-  const double a = 0.5 * w;
-  for (int64_t k = 0; k < nk; ++k) {
-    double s = 0;
+// Gauss-Legendre rule for the transform of the spreading kernel on [0, w/2]:
+// nodes and weight x phi, the same for every grid of a plan (phi is even, and
+// the ES kernel has a square-root edge, so there are many nodes).
+struct PhihatRule {
+  double a;
+  std::vector<double> z, wphi;
+  PhihatRule(int kind, int w, double beta) : a(0.5 * w) {
+    const int q = 8 * w + 64;
+    std::vector<double> x, wt;
+    gauss_legendre(q, &x, &wt);
     for (int i = 0; i < q; ++i) {
-      double z = 0.5 * a * (x[i] + 1.0);  // map [-1,1] -> [0, a]
-      s += wt[i] * spread_phi(kind, w, beta, z) * std::cos(2.0 * M_PI * k * z / nf);
+      z.push_back(0.5 * a * (x[i] + 1.0));  // map [-1, 1] -> [0, a]
+      wphi.push_back(wt[i] * spread_phi(kind, w, beta, z[i]));
     }
-    out[k] = 2.0 * 0.5 * a * s;
   }
+  // phihat(k) = 2 * integral_0^{w/2} phi(z) cos(2 pi k z / nf) dz, k = 0 .. nk-1
+  void table(int64_t nf, int64_t nk, double* out) const {
+    std::fill(out, out + nk, 0.0);
+    for (size_t i = 0; i < z.size(); ++i) {
+      // cos(k t) by rotation, started afresh every eight steps
+      const double t = 2.0 * M_PI * z[i] / double(nf), ct = std::cos(t), st = std::sin(t);
+      double c = 1.0, s = 0.0;
+      for (int64_t k = 0; k < nk; ++k) {
+        if ((k & 7) == 0) {
+          c = std::cos(2.0 * M_PI * double(k) * z[i] / double(nf));
+          s = std::sin(2.0 * M_PI * double(k) * z[i] / double(nf));
+        }
+        out[k] += wphi[i] * c;
+        const double cn = c * ct - s * st;
+        s = s * ct + c * st;
+        c = cn;
+      }
+    }
+    for (int64_t k = 0; k < nk; ++k) out[k] *= 2.0 * 0.5 * a;
+  }
+};
+
+void spread_phihat(int kind, int w, double beta, int64_t nf, int64_t nk, double* out) {
+  PhihatRule(kind, w, beta).table(nf, nk, out);
 }
 
 static bool spd_inverse(int d, const double* H, double* Hinv, double* det) {
@@ -493,11 +517,12 @@ fkreg_status compute_geometry(const fkreg_opts* o, fkreg_geometry* g, std::strin
   // 1/phihat tables: type-1 per axis, then per bandwidth per axis (k >= 0 half)
   if (tab) {
     tab->clear();
+    const PhihatRule rule(o->spread_kernel, w, beta);
     for (int j = 0; j < d; ++j) {
       phi1_off[j] = int64_t(tab->size());
       int64_t nk = g->modes[j] / 2;
       std::vector<double> ph(nk);
-      spread_phihat(o->spread_kernel, w, beta, g->nf[j], nk, ph.data());
+      rule.table(g->nf[j], nk, ph.data());
       for (int64_t k = 0; k < nk; ++k) tab->push_back(1.0 / ph[k]);
     }
     for (int b = 0; b < nbw; ++b)
@@ -505,7 +530,7 @@ fkreg_status compute_geometry(const fkreg_opts* o, fkreg_geometry* g, std::strin
         bws[b].phi2_off[j] = int64_t(tab->size());
         int64_t nk = bws[b].K[j] / 2;
         std::vector<double> ph(nk);
-        spread_phihat(o->spread_kernel, w, beta, bws[b].nf[j], nk, ph.data());
+        rule.table(bws[b].nf[j], nk, ph.data());
         for (int64_t k = 0; k < nk; ++k) tab->push_back(1.0 / ph[k]);
       }
   }
