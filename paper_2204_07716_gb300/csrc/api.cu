@@ -311,7 +311,10 @@ fkreg_status fkreg_plan_create(const fkreg_opts* opts, int64_t max_n, fkreg_plan
     t2_cells = std::max(t2_cells, full_cells(B.nf, d));
     t2_half = std::max(t2_half, half_cells(B.nf, d));
   }
-  const int64_t ntiles = (max_n + fk::kSortTileKeys - 1) / fk::kSortTileKeys;
+  // tiles of the sort for any n <= max_n
+  const int64_t ntiles = std::max<int64_t>(
+      (max_n + fk::kSortTileKeys - 1) / fk::kSortTileKeys,
+      (std::min<int64_t>(max_n, fk::kSmallTileMaxN) + fk::kSmallTile - 1) / fk::kSmallTile);
   const int64_t scan_len = std::max<int64_t>(1024 * ntiles, nb + 1);  // up to 10-bit digits
   Layout L;
   L.take(P->r_err, 256);

@@ -23,6 +23,11 @@ constexpr int kSubMin = 256;
 constexpr int kSubMax = 1024;
 constexpr int kRadixBits = 8;
 constexpr int kSortTileKeys = 4096;  // keys per radix-sort tile (one block)
+// Up to 512 tiles' worth of samples the fused sort takes tiles of 1024 keys: a
+// scatter is bound by the serial work of one block (16 rounds of 4096 keys), so
+// a small problem is as slow as a large one unless its keys go to more blocks.
+constexpr int kSmallTile = 1024;
+constexpr int64_t kSmallTileMaxN = 512 * kSmallTile;
 constexpr uint32_t kDefaultWaitLimit = 1u << 22;  // polls of a staged-window wait
 
 // Polynomials of the spreading kernel's inner taps (phi_row), tap k at distance

@@ -126,7 +126,7 @@ constexpr int64_t kFusedMaxBins = 8192;
 constexpr int kKeysThreads = 512;
 constexpr int kDigitScanWarps = 8;
 
-template <typename T, int B>
+template <typename T, int B, int TILE>
 __global__ void __launch_bounds__(kKeysThreads)
 keys_tiles_kernel(GeoDev g, int64_t n, int64_t nbins, int64_t ntiles, const T* __restrict__ x,
                   uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
@@ -141,8 +141,8 @@ keys_tiles_kernel(GeoDev g, int64_t n, int64_t nbins, int64_t ntiles, const T* _
   for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
     for (uint32_t d = threadIdx.x; d < R; d += blockDim.x) hd[d] = 0;
     __syncthreads();
-    const int64_t base = t * kSortTile;
-    for (int k = threadIdx.x; k < kSortTile; k += blockDim.x) {
+    const int64_t base = t * TILE;
+    for (int k = threadIdx.x; k < TILE; k += blockDim.x) {
       const int64_t i = base + k;
       if (i >= n) break;
       uint32_t bin;
@@ -386,7 +386,7 @@ __global__ void scan_apply(const uint32_t* in, int64_t n, const uint32_t* __rest
 }
 
 // ---- radix sort passes ---------------------------------------------------
-// A tile of kSortTile keys is split into one contiguous chunk per warp.  Both
+// A tile of keys is split into one contiguous chunk per warp.  Both
 // kernels group equal digits of a 32-key round with match_digit, so one
 // lane per group updates a counter: the upsweep adds to the tile histogram
 // (shared atomics, warps run concurrently); the downsweep first counts per
@@ -452,38 +452,38 @@ struct DownExtra {
   void* xs;
 };
 
-// dynamic shared memory of radix_downsweep<B, ...>
-template <int B>
+// dynamic shared memory of radix_downsweep<B, ..., TILE>
+template <int B, int TILE = kSortTile>
 constexpr size_t radix_down_smem() {
   return sizeof(uint32_t) * ((kSortThreads / 32 + 3) * (size_t(1) << B) + kSortThreads / 32 +
-                             2 * size_t(kSortTile));
+                             2 * size_t(TILE));
 }
 
-template <int B, int MODE = kDownPlain, typename T = float>
+template <int B, int MODE = kDownPlain, typename T = float, int TILE = kSortTile>
 __global__ void __launch_bounds__(kSortThreads, 2)
 radix_downsweep(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__ vals_in,
                 int64_t n, int shift, int64_t ntiles, const uint32_t* __restrict__ hist_scanned,
                 uint32_t* __restrict__ keys_out, uint32_t* __restrict__ vals_out, DownExtra ex) {
   constexpr int NW = kSortThreads / 32;
-  constexpr int RW = kSortTile / NW / 32;  // rounds of 32 keys per warp
+  constexpr int RW = TILE / NW / 32;  // rounds of 32 keys per warp
   constexpr uint32_t R = 1u << B;
   constexpr int DPT = int(R) / kSortThreads;  // digits per thread
-  static_assert(RW * NW * 32 == kSortTile && DPT >= 1 && DPT * kSortThreads == int(R),
+  static_assert(RW * NW * 32 == TILE && DPT >= 1 && DPT * kSortThreads == int(R),
                 "tile and digit layout");
   extern __shared__ __align__(16) uint32_t dsm[];
   uint32_t* wh = dsm;                  // [NW][R] per-warp counts, then offsets in the digit's run
   uint32_t* dstart = wh + NW * R;      // [R] first tile position of each digit
   uint32_t* gbase = dstart + R;        // [R] first output position of each digit
   uint32_t* wsum = gbase + R;          // [NW]
-  uint32_t* skey = wsum + NW;          // [kSortTile]
-  uint32_t* sval = skey + kSortTile;   // [kSortTile]
-  uint32_t* hn = sval + kSortTile;     // [R] next pass's digit totals (kDownCount)
+  uint32_t* skey = wsum + NW;          // [TILE]
+  uint32_t* sval = skey + TILE;        // [TILE]
+  uint32_t* hn = sval + TILE;          // [R] next pass's digit totals (kDownCount)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (uint32_t d = tid; d < NW * R; d += kSortThreads) wh[d] = 0;
   if (MODE == kDownCount)
     for (uint32_t d = tid; d < R; d += kSortThreads) hn[d] = 0;
   __syncthreads();
-  const int64_t tbase = int64_t(blockIdx.x) * kSortTile;
+  const int64_t tbase = int64_t(blockIdx.x) * TILE;
   const int64_t wbase = tbase + int64_t(warp) * (RW * 32);
   const uint32_t lt_mask = (1u << lane) - 1u;
   uint32_t key[RW], val[RW];
@@ -555,7 +555,7 @@ radix_downsweep(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
   __syncthreads();
   // write out in tile order: consecutive threads write consecutive positions
   // of one digit's run
-  const int cnt = int(n - tbase < kSortTile ? n - tbase : kSortTile);
+  const int cnt = int(n - tbase < TILE ? n - tbase : TILE);
   for (int t = tid; t < cnt; t += kSortThreads) {
     const uint32_t k = skey[t];
     const uint32_t dig = (k >> shift) & (R - 1u);
@@ -566,7 +566,7 @@ radix_downsweep(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
     if (MODE != kDownLast) keys_out[pos] = k;
     if (MODE == kDownCount) {
       const uint32_t dn = (k >> (shift + B)) & (R - 1u);
-      const int64_t hx = int64_t(dn) * ntiles + pos / uint32_t(kSortTile);
+      const int64_t hx = int64_t(dn) * ntiles + pos / uint32_t(TILE);
       if (in_range(ex.g.errw, kSiteSortHist, hx, int64_t(R) * ntiles)) atomicAdd(&ex.hist_next[hx], 1u);
       atomicAdd(&hn[dn], 1u);
     }
@@ -702,10 +702,11 @@ cudaError_t radix_pass(const uint32_t* kin, const uint32_t* vin, int64_t n, int 
 namespace {
 
 // The fused sort: keys_tiles, then per pass digit_scan and a scatter.
-template <int B, typename T>
-cudaError_t run_sort_fused(fkreg_plan_s* P, int64_t n, const T* x, int passes, int64_t ntiles,
+template <int B, int TILE, typename T>
+cudaError_t run_sort_fused(fkreg_plan_s* P, int64_t n, const T* x, int passes,
                            cudaStream_t s) {
   const GeoDev& g = P->geo;
+  const int64_t ntiles = (n + TILE - 1) / TILE;
   const int64_t nbins = P->nbins_total;
   uint32_t* keys[2] = {wsp<uint32_t>(P, P->r_keys0), wsp<uint32_t>(P, P->r_keys1)};
   uint32_t* vals[2] = {wsp<uint32_t>(P, P->r_vals0), wsp<uint32_t>(P, P->r_vals1)};
@@ -718,12 +719,12 @@ cudaError_t run_sort_fused(fkreg_plan_s* P, int64_t n, const T* x, int passes, i
   if (e != cudaSuccess) return e;
   const unsigned kb = unsigned(std::min<int64_t>(ntiles, int64_t(P->sm_count) * 2));
   const size_t ks = sizeof(uint32_t) * (size_t(nbins) + (size_t(1) << B));
-  keys_tiles_kernel<T, B><<<kb, kKeysThreads, ks, s>>>(g, n, nbins, ntiles, x, keys[0], vals[0],
+  keys_tiles_kernel<T, B, TILE><<<kb, kKeysThreads, ks, s>>>(g, n, nbins, ntiles, x, keys[0], vals[0],
                                                        counts, hist[0], dtot[0],
                                                        wsp<int>(P, P->r_err));
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   P->launches += 1;
-  constexpr size_t sm = radix_down_smem<B>();
+  constexpr size_t sm = radix_down_smem<B, TILE>();
   const BinsArgs bins{counts,
                       nbins,
                       g.sub_max,
@@ -743,18 +744,18 @@ cudaError_t run_sort_fused(fkreg_plan_s* P, int64_t n, const T* x, int passes, i
     DownExtra ex{last ? nullptr : hist[nx], last ? nullptr : dtot[nx], g, x,
                  wsp<T>(P, P->r_xs)};
     if (last) {
-      if ((e = cudaFuncSetAttribute(radix_downsweep<B, kDownLast, T>,
+      if ((e = cudaFuncSetAttribute(radix_downsweep<B, kDownLast, T, TILE>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm))) !=
           cudaSuccess)
         return e;
-      radix_downsweep<B, kDownLast, T><<<unsigned(ntiles), kSortThreads, sm, s>>>(
+      radix_downsweep<B, kDownLast, T, TILE><<<unsigned(ntiles), kSortThreads, sm, s>>>(
           keys[cur], vals[cur], n, p * B, ntiles, hist[p & 1], keys[cur ^ 1], vals[cur ^ 1], ex);
     } else {
-      if ((e = cudaFuncSetAttribute(radix_downsweep<B, kDownCount, T>,
+      if ((e = cudaFuncSetAttribute(radix_downsweep<B, kDownCount, T, TILE>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm))) !=
           cudaSuccess)
         return e;
-      radix_downsweep<B, kDownCount, T><<<unsigned(ntiles), kSortThreads, sm, s>>>(
+      radix_downsweep<B, kDownCount, T, TILE><<<unsigned(ntiles), kSortThreads, sm, s>>>(
           keys[cur], vals[cur], n, p * B, ntiles, hist[p & 1], keys[cur ^ 1], vals[cur ^ 1], ex);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -781,11 +782,16 @@ cudaError_t run_sort(fkreg_plan_s* P, int64_t n, const void* x, cudaStream_t s) 
   const int passes = (bits + dbits - 1) / dbits;
   if (n > 0 && passes >= 1 && nbins <= kFusedMaxBins) {
     const bool f32 = P->prec == FKREG_F32;
-    if (dbits == 10)
-      return f32 ? run_sort_fused<10>(P, n, static_cast<const float*>(x), passes, ntiles, s)
-                 : run_sort_fused<10>(P, n, static_cast<const double*>(x), passes, ntiles, s);
-    return f32 ? run_sort_fused<8>(P, n, static_cast<const float*>(x), passes, ntiles, s)
-               : run_sort_fused<8>(P, n, static_cast<const double*>(x), passes, ntiles, s);
+#define FK_FUSED(BB, TT)                                                                  \
+  return f32 ? run_sort_fused<BB, TT>(P, n, static_cast<const float*>(x), passes, s)      \
+             : run_sort_fused<BB, TT>(P, n, static_cast<const double*>(x), passes, s)
+    if (n <= kSmallTileMaxN) {
+      if (dbits == 10) FK_FUSED(10, kSmallTile);
+      FK_FUSED(8, kSmallTile);
+    }
+    if (dbits == 10) FK_FUSED(10, kSortTile);
+    FK_FUSED(8, kSortTile);
+#undef FK_FUSED
   }
   uint32_t* keys0 = wsp<uint32_t>(P, P->r_keys0);
   uint32_t* vals0 = wsp<uint32_t>(P, P->r_vals0);
