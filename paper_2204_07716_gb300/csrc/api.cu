@@ -291,7 +291,7 @@ fkreg_status fkreg_plan_create(const fkreg_opts* opts, int64_t max_n, fkreg_plan
     return set_global_error(FKREG_ERR_CUDA, "no CUDA device");
   }
   P->nblk_interp = int64_t(P->sm_count) * 8;
-  P->geo.sub_max = fk::sub_problem_size(d, P->prec == FKREG_F64, nb, max_n, P->sm_count);
+  P->geo.sub_max = fk::sub_problem_size(d, P->geo.w, P->prec == FKREG_F64, nb, max_n, P->sm_count);
   P->nsub_max = nb + (max_n + P->geo.sub_max - 1) / P->geo.sub_max;
   // tile + halo must fit shared memory for one strength
   {

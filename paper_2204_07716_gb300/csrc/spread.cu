@@ -5,10 +5,11 @@
 // sorted samples of one bin, accumulated into a shared-memory copy of the
 // bin's tile plus a halo of ceil(w/2) cells per side; the CTA then adds the
 // tile to the fine grid in global memory with one atomic per non-zero cell.
-// Two kernels fill the tile.  1-D and 2-D plans of a compile-time width use
+// Three kernels fill the tile.  1-D and 2-D plans of a compile-time width use
 // spread_run_kernel: the lanes of a warp cover the window cells and sum runs
 // of consecutive samples that share a window (the sort puts them together)
-// in registers before one shared-memory atomic per cell and strength.  3-D
+// in registers before one shared-memory atomic per cell and strength.  3-D FP32
+// plans of width 7 use spread_win3_kernel (the same, plane by plane).  FP64 3-D
 // and runtime widths use spread_kernel: each thread adds one sample's w^d
 // window at a time.  Strengths go in chunks that fit the shared-memory
 // budget.
@@ -400,6 +401,185 @@ spread_run_kernel(GeoDev g, int64_t n, const T* __restrict__ xs, const T* __rest
   }
 }
 
+// 3-D spreading of FP32 plans of width W: lanes over the window cells.
+//
+// A thread per sample (spread_kernel) met three costs here: neighbouring
+// samples of a warp hit the same cells and banks (2.8 atomics a clock and SM
+// of 32), a bin of 146 samples left 110 of the block's threads idle, and the
+// flush of its 24^3 cells took three runtime divisions a cell, more
+// instructions than the samples.  Here a warp takes a run of the bin's
+// samples, staged kNs at a time (kernel values, window origin, scaled
+// strength), and walks them with its lanes over the W x W cells of the last
+// two window axes; the W planes of sums stay in registers and go to the tile
+// when the window changes.  Tile rows are win3_pitch words apart, so that the
+// 32 cells of a step fall on (nearly) 32 banks, and the flush adds four cells
+// with one vector reduction.  All strengths are rows of one launch.
+// Measured on a GB300: 300,001 samples, two strengths on 120 x 90 x 100 cells
+// 250 -> 110 us (148 us with sub-problems of 1024 samples, see
+// sub_problem_size); 10^6 samples on 300^3 cells 313 -> 165 us a strength (263 us
+// with scalar reductions: 12,167 cells a bin, 83 times its samples, so the flush
+// and the clearing of the tile bound it now; the first case is bound by the issue
+// of conversions and tile atomics).
+constexpr int kNs = 16;  // samples staged per warp: 8 warps' rows and a 16^3 bin's tile fit three times
+
+// Rows W cells long and pitch = +-W mod 32 apart tile the banks.
+inline int win3_pitch(int w3, int w) {
+  while (w3 % 32 != w && w3 % 32 != 32 - w) ++w3;
+  return w3;
+}
+
+template <int W>
+__global__ void __launch_bounds__(kSpreadThreads, 3)
+spread_win3_kernel(GeoDev g, int64_t n, int pitch, const float* __restrict__ xs,
+                   const float* __restrict__ str, int s0, const uint32_t* __restrict__ sub_bin,
+                   const uint32_t* __restrict__ sub_first, const uint32_t* __restrict__ bin_start,
+                   const uint32_t* __restrict__ sub_total, float* __restrict__ fine) {
+  constexpr int CS = (W * W + 31) / 32;
+  constexpr int NWARP = kSpreadThreads / 32;
+  constexpr int PS = 3 * W;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ float s_red[NWARP];
+  __shared__ float s_phi[NWARP][kNs * PS], s_str[NWARP][kNs];
+  __shared__ int s_org[NWARP][kNs * 3];
+  int* sm = reinterpret_cast<int*>(smem_raw);
+  const uint32_t k = blockIdx.x;
+  if (k >= *sub_total) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t b = sub_bin[k];
+  const uint32_t first = sub_first[k];
+  const uint32_t last = min(first + g.sub_max, bin_start[b + 1]);
+  const int sc = s0 + int(blockIdx.y);
+  const float* c = str + int64_t(sc) * n;
+  int64_t o[3];
+  int W3[3];
+  {
+    uint32_t rem = b;
+#pragma unroll
+    for (int j = 2; j >= 0; --j) {
+      const uint32_t nb = uint32_t(g.nbins[j]);
+      const uint32_t q = rem / nb;
+      o[j] = int64_t(rem - q * nb) * g.tile[j] - g.pad;
+      W3[j] = int(g.tile[j]) + 2 * g.pad;
+      rem = q;
+    }
+  }
+  const int plane = W3[1] * pitch, words = W3[0] * plane;
+  for (int idx = threadIdx.x; idx < words; idx += kSpreadThreads) sm[idx] = 0;
+  // fixed-point scale: 2^30 / sum |c| over this sub-problem
+  float part = 0.f;
+  for (uint32_t p = first + threadIdx.x; p < last; p += kSpreadThreads) part += fabsf(c[p]);
+  part = warp_sum_t<float>(part);
+  if (lane == 0) s_red[warp] = part;
+  __syncthreads();
+  float tot = 0.f;
+#pragma unroll
+  for (int wv = 0; wv < NWARP; ++wv) tot += s_red[wv];
+  const float scale = tot > 0.f ? 1073741824.0f / tot : 0.f;
+  const float inv = tot > 0.f ? tot / 1073741824.0f : 0.f;
+  const float beta = float(g.beta), halfw = 0.5f * float(W);
+  // this lane's cells of a window plane
+  int rel[CS], c1[CS], c2[CS];
+  bool act[CS];
+#pragma unroll
+  for (int a = 0; a < CS; ++a) {
+    const int ci = lane + 32 * a;
+    act[a] = ci < W * W;
+    c1[a] = act[a] ? W + ci / W : 0;
+    c2[a] = act[a] ? 2 * W + ci % W : 0;
+    rel[a] = act[a] ? ci / W * pitch + ci % W : 0;
+  }
+  const int spare = words + lane;  // where lanes without a cell add
+  float acc[W][CS];
+#pragma unroll
+  for (int t = 0; t < W; ++t)
+#pragma unroll
+    for (int a = 0; a < CS; ++a) acc[t][a] = 0.f;
+  auto flush = [&](int cur) {
+#pragma unroll
+    for (int t = 0; t < W; ++t)
+#pragma unroll
+      for (int a = 0; a < CS; ++a) {
+        const int cell = act[a] ? cur + t * plane + rel[a] : spare;
+        if (in_range(g.errw, kSiteSpreadTile, cell, words + 32))
+          atomicAdd(&sm[cell], __float2int_rn(acc[t][a]));
+        acc[t][a] = 0.f;
+      }
+  };
+  const uint32_t len = last - first;
+  const uint32_t w_end = first + uint32_t(uint64_t(len) * (warp + 1) / NWARP);
+  int cur = -1;
+  for (uint32_t p0 = first + uint32_t(uint64_t(len) * warp / NWARP); p0 < w_end; p0 += kNs) {
+    const int cnt = int(min(uint32_t(kNs), w_end - p0));
+    for (int e = lane; e < 3 * cnt; e += 32) {  // one (sample, axis) per lane
+      const int j = e / 3, ax = e - 3 * j;
+      const float u = mul_rn(xs[int64_t(ax) * n + p0 + j],
+                             ax == 0 ? inv_h_of<float>(g, 0)
+                                     : (ax == 1 ? inv_h_of<float>(g, 1) : inv_h_of<float>(g, 2)));
+      const float f0 = ceilf(u - halfw);
+      const int l = int(int64_t(f0) - (ax == 0 ? o[0] : (ax == 1 ? o[1] : o[2])));
+      s_org[warp][e] = l * (ax == 0 ? plane : (ax == 1 ? pitch : 1));
+#pragma unroll
+      for (int t = 0; t < W; ++t)
+        s_phi[warp][j * PS + ax * W + t] = phi<float>(g.skind, W, beta, f0 - u + float(t));
+    }
+    if (lane < cnt) s_str[warp][lane] = c[p0 + lane] * scale;
+    __syncwarp();
+#pragma unroll 2
+    for (int j = 0; j < cnt; ++j) {
+      const int org = s_org[warp][3 * j] + s_org[warp][3 * j + 1] + s_org[warp][3 * j + 2];
+      if (org != cur) {
+        if (cur >= 0) flush(cur);
+        cur = org;
+      }
+      const float* ph = s_phi[warp] + j * PS;
+      const float cv = s_str[warp][j];
+      float p[CS];
+#pragma unroll
+      for (int a = 0; a < CS; ++a) p[a] = cv * (ph[c1[a]] * ph[c2[a]]);
+#pragma unroll
+      for (int t = 0; t < W; ++t) {
+        const float w0 = ph[t];
+#pragma unroll
+        for (int a = 0; a < CS; ++a) acc[t][a] = fmaf(w0, p[a], acc[t][a]);
+      }
+    }
+    __syncwarp();  // the staging rows are rewritten
+  }
+  if (cur >= 0) flush(cur);
+  __syncthreads();
+  // flush the tile (periodic wrap): quads of cells in one vector reduction each
+  // where the tiles start and wrap on multiples of four cells
+  const int64_t fine_cells = g.nf[0] * g.nf[1] * g.nf[2];
+  float* out = fine + int64_t(sc) * fine_cells;
+  const bool quads = (g.nf[2] & 3) == 0 && (o[2] & 3) == 0 && (W3[2] & 3) == 0 && W3[2] <= 128;
+  const int qn = quads ? W3[2] >> 2 : 32, rows = 32 / qn;  // rows of one warp step
+  const int sub = lane / qn, q = lane - sub * qn;
+  int l0 = 0, l1 = warp * rows + sub;
+  for (int row = l1; row < W3[0] * W3[1]; row += NWARP * rows, l1 += NWARP * rows) {
+    if (sub >= rows) break;
+    while (l1 >= W3[1]) {
+      l1 -= W3[1];
+      ++l0;
+    }
+    const int64_t r = (wrap_idx(o[0] + l0, g.nf[0]) * g.nf[1] + wrap_idx(o[1] + l1, g.nf[1])) * g.nf[2];
+    const int* src = sm + l0 * plane + l1 * pitch;
+    if (quads) {
+      const int4 v = make_int4(src[4 * q], src[4 * q + 1], src[4 * q + 2], src[4 * q + 3]);
+      const int64_t gi = r + wrap_idx(o[2] + 4 * q, g.nf[2]);
+      if ((v.x | v.y | v.z | v.w) != 0 && in_range(g.errw, kSiteSpreadFlush, gi + 3, fine_cells))
+        atomicAdd(reinterpret_cast<float4*>(out + gi),
+                  make_float4(float(v.x) * inv, float(v.y) * inv, float(v.z) * inv, float(v.w) * inv));
+    } else {
+      for (int l2 = lane; l2 < W3[2]; l2 += 32) {
+        const int v = src[l2];
+        const int64_t gi = r + wrap_idx(o[2] + l2, g.nf[2]);
+        if (v != 0 && in_range(g.errw, kSiteSpreadFlush, gi, fine_cells))
+          atomicAdd(&out[gi], float(v) * inv);
+      }
+    }
+  }
+}
+
 template <typename T, int D, int W, int CN>
 cudaError_t launch_spread_cn(fkreg_plan_s* P, int s0, cudaStream_t st) {
   const GeoDev& g = P->geo;
@@ -497,6 +677,26 @@ cudaError_t launch_spread_runs(fkreg_plan_s* P, int s0, int scount, cudaStream_t
   return cudaSuccess;
 }
 
+// All strengths in one launch, a grid row each.
+cudaError_t launch_spread_win3(fkreg_plan_s* P, int s0, int scount, cudaStream_t st, bool* launched) {
+  const GeoDev& g = P->geo;
+  const int pitch = win3_pitch(int(g.tile[2]) + 2 * g.pad, 7);
+  const size_t smem = sizeof(int) * size_t(g.tile[0] + 2 * g.pad) * size_t(g.tile[1] + 2 * g.pad) * pitch +
+                      32 * sizeof(int);
+  if (smem > 200 * 1024 || scount > 65535) return cudaSuccess;
+  *launched = true;
+  cudaError_t e = cudaFuncSetAttribute(spread_win3_kernel<7>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  if (e != cudaSuccess) return e;
+  const uint32_t* sub_total = wsp<uint32_t>(P, P->r_substart) + P->nbins_total;
+  spread_win3_kernel<7><<<dim3(unsigned(P->nsub_max), unsigned(scount)), kSpreadThreads, smem, st>>>(
+      g, P->n, pitch, wsp<float>(P, P->r_xs), wsp<float>(P, P->r_str), s0,
+      wsp<uint32_t>(P, P->r_subbin), wsp<uint32_t>(P, P->r_subfirst),
+      wsp<uint32_t>(P, P->r_binstart), sub_total, wsp<float>(P, P->r_fine));
+  P->launches += 1;
+  return cudaGetLastError();
+}
+
 // Strengths go in launches of 8, 4, 2 or 1 (compile-time chunk sizes, as
 // many as the shared-memory budget allows per launch); 1-D / 2-D plans of a
 // compile-time width use the run kernel instead (launch_spread_runs).
@@ -505,6 +705,11 @@ cudaError_t launch_spread_w(fkreg_plan_s* P, int s0, int scount, cudaStream_t st
   const GeoDev& g = P->geo;
   if constexpr (W > 0 && D <= 2) {
     if (spread_run_smem<T, D, W, 1>(g) <= 220 * 1024) return launch_spread_runs<T, D, W>(P, s0, scount, st);
+  }
+  if constexpr (sizeof(T) == 4 && W == 7 && D == 3) {
+    bool launched = false;
+    const cudaError_t e = launch_spread_win3(P, s0, scount, st, &launched);
+    if (launched || e != cudaSuccess) return e;
   }
   int cells = 1;
   for (int j = 0; j < D; ++j) cells *= int(g.tile[j]) + 2 * g.pad;
