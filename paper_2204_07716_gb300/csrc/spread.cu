@@ -225,11 +225,13 @@ spread_kernel(GeoDev g, int64_t n, const T* __restrict__ xs, const T* __restrict
 // window in registers and adds them to the tile only when the window changes;
 // the sort puts samples that share a window next to each other, so the
 // shared-memory atomics drop from one per sample, cell and strength to one
-// per run of samples, cell and strength.
-template <typename T, int D, int W, int CN>
+// per run of samples, cell and strength.  One launch takes CN strengths from s0
+// on; with RAG it takes the ncn < CN there are and repeats the last one in sums
+// that are not flushed (a test for each strength instead cost 15 % of full launches).
+template <typename T, int D, int W, int CN, bool RAG>
 __global__ void __launch_bounds__(kSpreadThreads)
 spread_run_kernel(GeoDev g, int64_t n, const T* __restrict__ xs, const T* __restrict__ str,
-                  int s0, const uint32_t* __restrict__ sub_bin,
+                  int s0, int ncn, const uint32_t* __restrict__ sub_bin,
                   const uint32_t* __restrict__ sub_first, const uint32_t* __restrict__ bin_start,
                   const uint32_t* __restrict__ sub_total, T* __restrict__ fine,
                   PhiTab<T> tab) {
@@ -282,7 +284,7 @@ spread_run_kernel(GeoDev g, int64_t n, const T* __restrict__ xs, const T* __rest
     for (int c = 0; c < CN; ++c) part[c] = T(0);
     for (uint32_t p = first + threadIdx.x; p < last; p += blockDim.x)
 #pragma unroll
-      for (int c = 0; c < CN; ++c) part[c] += fabs(str[int64_t(s0 + c) * n + p]);
+      for (int c = 0; c < CN; ++c) part[c] += fabs(str[int64_t(s0 + (RAG ? min(c, ncn - 1) : c)) * n + p]);
 #pragma unroll
     for (int c = 0; c < CN; ++c) {
       const T v = warp_sum_t<T>(part[c]);
@@ -330,7 +332,8 @@ spread_run_kernel(GeoDev g, int64_t n, const T* __restrict__ xs, const T* __rest
       }
       org_row[lane] = org;
 #pragma unroll
-      for (int c = 0; c < CN; ++c) str_rows[lane * CN + c] = str[int64_t(s0 + c) * n + p] * s_scale[c];
+      for (int c = 0; c < CN; ++c)
+        str_rows[lane * CN + c] = str[int64_t(s0 + (RAG ? min(c, ncn - 1) : c)) * n + p] * s_scale[c];
     }
     __syncwarp();
     T acc[CS][CN];
@@ -394,7 +397,7 @@ spread_run_kernel(GeoDev g, int64_t n, const T* __restrict__ xs, const T* __rest
     int64_t gidx = wrap_idx(o[0] + l0, g.nf[0]);
     if (D == 2) gidx = gidx * g.nf[1] + wrap_idx(o[1] + l1, g.nf[1]);
     if (!in_range(g.errw, kSiteSpreadFlush, gidx, fine_cells)) continue;
-    for (int c = 0; c < CN; ++c) {
+    for (int c = 0; c < (RAG ? ncn : CN); ++c) {
       const A av = sm[c * cells + idx];
       if (av != A(0)) atomicAdd(&fine[int64_t(s0 + c) * fine_cells + gidx], T(av) * s_inv[c]);
     }
@@ -620,59 +623,65 @@ PhiTab<T> phi_tab(const fkreg_plan_s* P) {
     return {};
 }
 
-template <typename T, int D, int W, int CN>
-cudaError_t launch_spread_run(fkreg_plan_s* P, int s0, cudaStream_t st) {
+template <typename T, int D, int W, int CN, bool RAG>
+cudaError_t launch_spread_run(fkreg_plan_s* P, int s0, int ncn, cudaStream_t st) {
   const GeoDev& g = P->geo;
   const size_t smem = spread_run_smem<T, D, W, CN>(g);
   if (smem > 220 * 1024) return cudaErrorInvalidConfiguration;
-  cudaError_t e = cudaFuncSetAttribute(spread_run_kernel<T, D, W, CN>,
+  cudaError_t e = cudaFuncSetAttribute(spread_run_kernel<T, D, W, CN, RAG>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
   const unsigned grid = unsigned(P->nsub_max);
   const uint32_t* sub_total = wsp<uint32_t>(P, P->r_substart) + P->nbins_total;
-  spread_run_kernel<T, D, W, CN><<<grid, kSpreadThreads, smem, st>>>(
-      g, P->n, wsp<T>(P, P->r_xs), wsp<T>(P, P->r_str), s0, wsp<uint32_t>(P, P->r_subbin),
+  spread_run_kernel<T, D, W, CN, RAG><<<grid, kSpreadThreads, smem, st>>>(
+      g, P->n, wsp<T>(P, P->r_xs), wsp<T>(P, P->r_str), s0, ncn, wsp<uint32_t>(P, P->r_subbin),
       wsp<uint32_t>(P, P->r_subfirst), wsp<uint32_t>(P, P->r_binstart), sub_total,
       wsp<T>(P, P->r_fine), phi_tab<T>(P));
   P->launches += 1;
   return cudaGetLastError();
 }
 
-// All strengths through the run kernel in launches of the largest chunk
-// sizes that fit shared memory (FP32: 16, 12, 8, 4, 2, 1; FP64: 4, 2, 1).
+// `ncn` strengths in one launch of the smallest instantiated size that holds
+// them (CN ascending over the sizes); *fits says whether its block fits.
+template <typename T, int D, int W, int CN, int... More>
+cudaError_t launch_spread_size(fkreg_plan_s* P, int s0, int ncn, cudaStream_t st, bool* fits) {
+  if constexpr (sizeof...(More) > 0)
+    if (ncn > CN) return launch_spread_size<T, D, W, More...>(P, s0, ncn, st, fits);
+  *fits = ncn <= CN && spread_run_smem<T, D, W, CN>(P->geo) <= 220 * 1024;
+  if (!*fits) return cudaSuccess;
+  if (ncn == CN) return launch_spread_run<T, D, W, CN, false>(P, s0, ncn, st);
+  if constexpr (CN > 2 && CN < 16) return launch_spread_run<T, D, W, CN, true>(P, s0, ncn, st);
+  return cudaErrorInvalidValue;
+}
+
+// All strengths through the run kernel (sizes: FP32 16, 12, 8, 4, 2, 1; FP64 4, 2,
+// 1).  A launch costs a fixed part (kernel values, staging, tile) and far less per
+// strength, so three, five to seven and nine to eleven strengths go in one launch
+// of the next size up.  Twelve strengths are four blocks an SM, sixteen are three:
+// FP32 2-D, 2 10^6 samples on 448 x 448 cells take 83, 95, 114, 178 and 254 us with 1,
+// 2, 4, 12 and 16, so larger counts go twelve at a time (39 strengths: 640 us,
+// 800 in launches of 16, 16, 4, 2 and 1).  Where a size does not fit shared memory
+// the next smaller ones are taken.
 template <typename T, int D, int W>
 cudaError_t launch_spread_runs(fkreg_plan_s* P, int s0, int scount, cudaStream_t st) {
-  int done = 0;
-  while (done < scount) {
+  constexpr bool f32 = sizeof(T) == 4;
+  int cap = f32 ? 16 : 4;
+  for (int done = 0; done < scount;) {
     const int rem = scount - done;
-    cudaError_t e = cudaErrorInvalidConfiguration;
-    int used = 0;
-    if constexpr (sizeof(T) == 4) {
-      if (rem >= 16 && spread_run_smem<T, D, W, 16>(P->geo) <= 220 * 1024) {
-        e = launch_spread_run<T, D, W, 16>(P, s0 + done, st);
-        used = 16;
-      } else if (rem >= 12 && spread_run_smem<T, D, W, 12>(P->geo) <= 220 * 1024) {
-        e = launch_spread_run<T, D, W, 12>(P, s0 + done, st);
-        used = 12;
-      } else if (rem >= 8 && spread_run_smem<T, D, W, 8>(P->geo) <= 220 * 1024) {
-        e = launch_spread_run<T, D, W, 8>(P, s0 + done, st);
-        used = 8;
-      }
-    }
-    if (!used) {
-      if (rem >= 4 && spread_run_smem<T, D, W, 4>(P->geo) <= 220 * 1024) {
-        e = launch_spread_run<T, D, W, 4>(P, s0 + done, st);
-        used = 4;
-      } else if (rem >= 2 && spread_run_smem<T, D, W, 2>(P->geo) <= 220 * 1024) {
-        e = launch_spread_run<T, D, W, 2>(P, s0 + done, st);
-        used = 2;
-      } else {
-        e = launch_spread_run<T, D, W, 1>(P, s0 + done, st);
-        used = 1;
-      }
-    }
+    const int used = std::min(rem, f32 && rem != 16 ? std::min(cap, 12) : cap);
+    bool fits = false;
+    cudaError_t e;
+    if constexpr (f32)
+      e = launch_spread_size<T, D, W, 1, 2, 4, 8, 12, 16>(P, s0 + done, used, st, &fits);
+    else
+      e = launch_spread_size<T, D, W, 1, 2, 4>(P, s0 + done, used, st, &fits);
     if (e != cudaSuccess) return e;
-    done += used;
+    if (fits)
+      done += used;
+    else if (used == 1)
+      return cudaErrorInvalidConfiguration;
+    else
+      cap = used > 12 ? 12 : (used > 8 ? 8 : (used > 4 ? 4 : (used > 2 ? 2 : 1)));
   }
   return cudaSuccess;
 }
