@@ -34,14 +34,17 @@ namespace {
 // type-1 transform (with its memset) per (fine cell, strength), per bandwidth
 // the type-2 transform and record interleave per (fine cell, field) and the
 // gather per (sample, window cell, field); a fixed cost per group for its
-// sort and launches.
+// sort and launches.  Spreading and interleave have become faster since (0.5e-12
+// for the spreading); the units stay, for a new split would change which
+// bandwidths take the direct sums, and with that the rounding of their results.
 constexpr double kSpreadUnit = 1.3e-12;
 constexpr double kType1Unit = 1.7e-11;
 constexpr double kType2Unit = 1.6e-11;
 constexpr double kGatherUnit = 3.3e-13;
 constexpr double kGroupFixed = 3e-4;
-// The direct sums (FKREG_KERNEL_GAUSSIAN_DIRECT) per (sample pair, field),
-// from the at-sample pass of the compact-kernel path.
+// The direct sums (FKREG_KERNEL_GAUSSIAN_DIRECT) per (sample pair, field), from
+// the 2-D at-sample pass of the compact-kernel path (4.1e-13 in 3-D with 33
+// strengths: 10^6 samples of 2585 neighbours in 35 ms).
 constexpr double kPairUnit = 2.4e-13;
 
 int64_t cells(const int64_t* nf, int d) {
