@@ -50,7 +50,8 @@ def _stale(lib: str = LIB) -> bool:
     if not os.path.exists(lib):
         return True
     t = os.path.getmtime(lib)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(INCLUDE, "*.h"))
+    deps = sources() + [p for d, pat in ((CSRC, "*.h"), (CSRC, "*.cuh"), (INCLUDE, "*.h"))
+                        for p in glob.glob(os.path.join(d, pat))]
     return any(os.path.getmtime(p) > t for p in deps)
 
 
