@@ -154,6 +154,7 @@ typedef struct {
  *              Fourier series, chosen so no wrap-around reaches the box
  *              (the role of the zero padding of eq. 18)
  *   ldft[j]    L_j, length of the inverse DFT onto the grid lattice (eq. 21)
+ *              (even on the last axis, but for 1-D plans of at most 4096)
  *   modes[j]   K_j, even; Fourier modes |k_j| <= K_j/2 - 1 are kept
  *   nf[j]      fine (oversampled) grid of the type-1 spreading, >= 2 K_j
  *   w, beta    spreading width in fine cells and ES shape parameter

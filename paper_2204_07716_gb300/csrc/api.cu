@@ -320,7 +320,7 @@ fkreg_status fkreg_plan_create(const fkreg_opts* opts, int64_t max_n, fkreg_plan
   L.take(P->r_err, 256);
   L.take(P->r_bw, sizeof(fk::BwDev) * P->nbw);
   L.take(P->r_tab, sizeof(double) * std::max<size_t>(1, P->tab.size()));
-  // 1-D transforms of up to 4096 points, odd ones beyond, are the library's own (fft1d.cu)
+  // 1-D transforms of up to 4096 points are the library's own (fft1d.cu)
   if (!P->direct && d == 1) {
     std::vector<int64_t> lens = {P->g.nf[0], P->g.ldft[0]};
     for (const auto& B : P->bw) lens.push_back(B.nf[0]);

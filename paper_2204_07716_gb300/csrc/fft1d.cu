@@ -1,5 +1,4 @@
-// Fourier transforms of 1-D plans up to 4096 points (odd lengths as far as a
-// block's shared memory holds them): one block per transform,
+// Fourier transforms of 1-D plans up to 4096 points: one block per transform,
 // mixed radix (4, 2, 3, 5, 7) Stockham passes in shared memory with a table of
 // the roots of unity that the plan computes once in FP64.
 //
@@ -220,14 +219,10 @@ cudaError_t launch(fkreg_plan_s* P, bool inverse, int64_t n, int batch, const vo
 }  // namespace
 
 // Lengths this file transforms: 7-smooth (every length of the planner is), two
-// copies of the points and their roots in a block's shared memory.  Past 4096
-// points one block is no longer quicker than cuFFT's many, but cuFFT's real
-// transforms of odd lengths lose four digits (FP32, 5103 points: a grid estimate
-// 5e-3 off; 1029 points: 2e-4; 3e-7 here), so odd lengths stay here as long as
-// they fit (9555 points in FP32, 4777 in FP64; a call of 5103 takes the same 70 us).
+// copies of the points and their roots in a block's shared memory (196 KB for 4096
+// points in FP64).  Past that one block is no longer quicker than cuFFT's many.
 bool fft1d_applies(const fkreg_plan_s* P, int64_t n) {
-  if (P->d != 1 || n < 2) return false;
-  if (n > 4096 && (n % 2 == 0 || 6 * size_t(n) * P->tsize > 224 * 1024)) return false;
+  if (P->d != 1 || n < 2 || n > kFft1dMax) return false;
   for (int r : {2, 3, 5, 7})
     while (n % r == 0) n /= r;
   return n == 1;

@@ -28,6 +28,7 @@ constexpr int kSortTileKeys = 4096;  // keys per radix-sort tile (one block)
 // a small problem is as slow as a large one unless its keys go to more blocks.
 constexpr int kSmallTile = 1024;
 constexpr int64_t kSmallTileMaxN = 512 * kSmallTile;
+constexpr int64_t kFft1dMax = 4096;  // longest 1-D transform of fft1d.cu
 constexpr uint32_t kDefaultWaitLimit = 1u << 22;  // polls of a staged-window wait
 
 // Polynomials of the spreading kernel's inner taps (phi_row), tap k at distance
