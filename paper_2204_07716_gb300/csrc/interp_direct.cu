@@ -9,7 +9,10 @@
 // on the tensor cores (mma_union_gather: split-TF32 products over the
 // union); other warps, and 1-D plans, gather lane per sample with packed FP32
 // FMAs.  The gather-only form (GONLY) writes V[f][s] for the backward instead
-// of phase B; the full form writes V beside phase B when it is given one.
+// of phase B; KEEP writes V beside phase B, for the GCV backward's forward
+// pass.  Every other pass is compiled without that store: with a test of the
+// pointer in it instead, 2-D local linear with 40 fields spills 60 / 68 bytes a
+// thread for 44 / 60 and with 48 fields 32 / 48 for none.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -28,7 +31,7 @@ namespace {
 template <int D>
 constexpr int direct_warps() { return D == 2 ? 12 : kLWarps; }
 
-template <int D, int W, int NQ, int ORD, bool GONLY>
+template <int D, int W, int NQ, int ORD, bool GONLY, bool KEEP>
 __global__ void __launch_bounds__(direct_warps<D>() * 32, 1)
 interp_direct_kernel(GeoDev g, const BwDev* __restrict__ bwt, int b, int64_t n,
                      const float* __restrict__ xs, const float* __restrict__ str,
@@ -234,7 +237,7 @@ interp_direct_kernel(GeoDev g, const BwDev* __restrict__ bwt, int b, int64_t n,
                                          acc);
         }
       }
-      if (GONLY || vout) {
+      if (GONLY || KEEP) {
         if (valid)
 #pragma unroll
           for (int q = 0; q < NQ; ++q)
@@ -355,12 +358,12 @@ interp_direct_kernel(GeoDev g, const BwDev* __restrict__ bwt, int b, int64_t n,
 }
 
 
-template <int D, int NQ, int ORD, bool GONLY>
+template <int D, int NQ, int ORD, bool GONLY, bool KEEP>
 cudaError_t launch_direct_k(fkreg_plan_s* P, int b, int n_rhs_real, int n_probes,
                             void* mhat_at_x, cudaStream_t st, int nacc, int F2, float* vout,
                             int rec, int wm0, int wm1, int pitch, int slack, int win_floats,
                             int nw, size_t smem, unsigned grid) {
-  auto kern = interp_direct_kernel<D, 7, NQ, ORD, GONLY>;
+  auto kern = interp_direct_kernel<D, 7, NQ, ORD, GONLY, KEEP>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
   kern<<<grid, nw * 32, smem, st>>>(
@@ -374,15 +377,15 @@ cudaError_t launch_direct_k(fkreg_plan_s* P, int b, int n_rhs_real, int n_probes
   return cudaGetLastError();
 }
 
-template <int D, int ORD, bool GONLY>
+template <int D, int ORD, bool GONLY, bool KEEP>
 cudaError_t launch_direct_q(fkreg_plan_s* P, int b, int n_rhs_real, int n_probes,
                             void* mhat_at_x, cudaStream_t st, int nacc, int F2, float* vout,
                             int rec, int wm0, int wm1, int pitch, int slack, int win_floats,
                             int nw, size_t smem, unsigned grid) {
 #define FK_Q(Q)                                                                                  \
-  return launch_direct_k<D, Q, ORD, GONLY>(P, b, n_rhs_real, n_probes, mhat_at_x, st, nacc, F2, \
-                                           vout, rec, wm0, wm1, pitch, slack, win_floats, nw,     \
-                                           smem, grid)
+  return launch_direct_k<D, Q, ORD, GONLY, KEEP>(P, b, n_rhs_real, n_probes, mhat_at_x, st,     \
+                                                 nacc, F2, vout, rec, wm0, wm1, pitch, slack,    \
+                                                 win_floats, nw, smem, grid)
   switch (interp_quads(F2)) {
     case 2: FK_Q(2);
     case 4: FK_Q(4);
@@ -435,19 +438,24 @@ cudaError_t run_interp_direct(fkreg_plan_s* P, int b, int n_rhs_real, int n_prob
   const unsigned grid = unsigned(std::min<int64_t>(P->sm_count, std::max<int64_t>(1, P->nsub_max)));
   float* vo = static_cast<float*>(vout);
   *launched = true;
-#define FK_A(DD, OO, GG)                                                                        \
-  return launch_direct_q<DD, OO, GG>(P, b, n_rhs_real, n_probes, mhat_at_x, st, nacc, F2, vo,  \
-                                     rec, wm0, wm1, pitch, slack, win_floats, nw, smem, grid)
+#define FK_A(DD, OO, GG, KK)                                                                     \
+  return launch_direct_q<DD, OO, GG, KK>(P, b, n_rhs_real, n_probes, mhat_at_x, st, nacc, F2,   \
+                                         vo, rec, wm0, wm1, pitch, slack, win_floats, nw, smem, \
+                                         grid)
   if (gonly) {
-    if (D == 1) FK_A(1, 0, true);
-    FK_A(2, 0, true);
+    if (D == 1) FK_A(1, 0, true, false);
+    FK_A(2, 0, true, false);
   }
-  if (D == 1) {
-    if (P->order == 0) FK_A(1, 0, false);
-    FK_A(1, 1, false);
+  if (vo) {
+    if (D == 1 && P->order == 0) FK_A(1, 0, false, true);
+    if (D == 1) FK_A(1, 1, false, true);
+    if (P->order == 0) FK_A(2, 0, false, true);
+    FK_A(2, 1, false, true);
   }
-  if (P->order == 0) FK_A(2, 0, false);
-  FK_A(2, 1, false);
+  if (D == 1 && P->order == 0) FK_A(1, 0, false, false);
+  if (D == 1) FK_A(1, 1, false, false);
+  if (P->order == 0) FK_A(2, 0, false, false);
+  FK_A(2, 1, false, false);
 #undef FK_A
 }
 
