@@ -357,6 +357,9 @@ fkreg_status fkreg_plan_create(const fkreg_opts* opts, int64_t max_n, fkreg_plan
   L.take(P->r_t2field,
          std::max<int64_t>(256, fft_scale * T * int64_t(fk::t2_record_stride(t2_fields, T)) * t2_cells));
   L.take(P->r_part, sizeof(double) * size_t(P->nblk_interp + 1) * P->nbw * P->nacc);
+  // direct path: sums of each group of 32 samples
+  const size_t ngroups = P->direct ? size_t(max_n + 31) / 32 : 0;
+  L.take(P->r_gsum, std::max<size_t>(256, sizeof(double) * P->nacc * ngroups));
   L.take(P->r_smax, 8 * size_t(P->nbw));
   if (P->backward) {
     const int64_t nn = std::max<int64_t>(1, max_n);

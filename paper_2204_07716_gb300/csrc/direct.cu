@@ -143,7 +143,6 @@ struct DsArgs {
   int fields;          // fields per target (ns + nstr nt)
   int str_pass;        // the strengths' pass (see kStrFlag)
   int64_t ntask;       // groups of 32 targets
-  int64_t nblk_rows;   // at samples: rows of partial sums to fill
   int64_t Mtot;        // grid: points
 };
 
@@ -220,7 +219,7 @@ __global__ void __launch_bounds__(kDsThreads)
 direct_sums_kernel(GeoDev g, MonoTab mono, DsArgs a, const BwDev* __restrict__ bwt, int64_t n,
                    const T* __restrict__ xs, const T* __restrict__ str,
                    const uint32_t* __restrict__ perm, const uint32_t* __restrict__ bin_start,
-                   T* __restrict__ field, T* __restrict__ mhat_at_x, double* __restrict__ part,
+                   T* __restrict__ field, T* __restrict__ mhat_at_x, double* __restrict__ gsum,
                    uint32_t* __restrict__ task_count) {
   constexpr int NS = mono_count(D, 2 * ORD), NT = mono_count(D, ORD), RS = ds_stride<QC>();
   using C4 = typename DsCoord<T>::type;
@@ -230,7 +229,7 @@ direct_sums_kernel(GeoDev g, MonoTab mono, DsArgs a, const BwDev* __restrict__ b
   __shared__ uint32_t s_qi[kDsWarps][64];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // layout: strengths [warps][32][RS], the warps' fields [warps][32][bstride],
-  // the reduction accumulators [nacc] (RS is a multiple of 4, the rows are 128)
+  // the group's reduction accumulators [nacc] (RS is a multiple of 4, the rows are 128)
   T* rec = reinterpret_cast<T*>(smem_raw) + warp * 32 * RS;
   T* rows_f = reinterpret_cast<T*>(smem_raw) + kDsThreads * RS;
   T* my = rows_f + tid * a.bstride;
@@ -251,8 +250,9 @@ direct_sums_kernel(GeoDev g, MonoTab mono, DsArgs a, const BwDev* __restrict__ b
   // some strength of this pass is not finite: it must not reach targets that
   // hold its sample outside their support through a product with zero
   const bool nonfin = g.errw[kStrFlag] == a.str_pass;
-  __shared__ uint32_t s_task;
+  __shared__ uint32_t s_task, s_row;
   for (int64_t task = blockIdx.x; task < a.ntask;) {
+    if (!GRID && tid == 0) s_row = uint32_t(task);
     // this lane's target, the same in all four warps
     T qv[D];
     bool valid;
@@ -465,22 +465,35 @@ direct_sums_kernel(GeoDev g, MonoTab mono, DsArgs a, const BwDev* __restrict__ b
       }
       // the groups of a dense region cost tens of times those of a sparse one: the
       // resident blocks take them from a counter (dealt out in turn, half the
-      // SMs idled through the second half of the pass)
+      // SMs idled through the second half of the pass).  Which block takes a group
+      // differs from run to run, so each group leaves its own row of sums
+      // (ds_rows_kernel adds them in a fixed order)
       if (tid == 0) s_task = gridDim.x + atomicAdd(task_count, 1u);
+      const uint32_t row = s_row;
       __syncthreads();  // also: the rows are rewritten by the next task
+      for (int k = tid; k < a.nacc; k += kDsThreads) {
+        gsum[int64_t(row) * a.nacc + k] = red_get<T>(red, k);
+        red[k] = 0.0;
+      }
       task = s_task;
     } else {
       break;  // one block per patch
     }
   }
-  if constexpr (!GRID) {
-    for (int k = tid; k < a.nacc; k += kDsThreads) {
-      part[(int64_t(blockIdx.x) * a.nbw + a.b) * a.nacc + k] = red_get<T>(red, k);
-      // partial rows of the block indices this one-wave grid does not launch
-      for (int64_t r = int64_t(blockIdx.x) + gridDim.x; r < a.nblk_rows; r += gridDim.x)
-        part[(r * a.nbw + a.b) * a.nacc + k] = 0.0;
-    }
-  }
+}
+
+// The rows of partial sums that the reduction reads, from the groups' sums: row r
+// adds groups r, r + rows, ... in turn, whichever block took them, so the scalars of
+// a call repeat bit for bit.
+__global__ void ds_rows_kernel(const double* __restrict__ gsum, int64_t ntask, int nacc, int nbw,
+                               int b, int64_t rows, double* __restrict__ part) {
+  const int64_t id = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (id >= rows * nacc) return;
+  const int64_t r = id / nacc;
+  const int k = int(id - r * nacc);
+  double t = 0.0;
+  for (int64_t i = r; i < ntask; i += rows) t += gsum[i * nacc + k];
+  part[(r * nbw + b) * nacc + k] = t;
 }
 
 template <typename T, int D, int ORD, int QC, bool GRID>
@@ -506,7 +519,13 @@ cudaError_t launch_ds(fkreg_plan_s* P, DsArgs a, int bw_count, void* mhat_at_x, 
   kern<<<dim3(unsigned(blocks), unsigned(bw_count)), kDsThreads, smem, st>>>(
       P->geo, P->mono, a, wsp<BwDev>(P, P->r_bw), P->n, wsp<T>(P, P->r_xs), wsp<T>(P, P->r_str),
       perm_ptr(P), wsp<uint32_t>(P, P->r_binstart), wsp<T>(P, P->r_gfield),
-      static_cast<T*>(mhat_at_x), wsp<double>(P, P->r_part), task_count);
+      static_cast<T*>(mhat_at_x), wsp<double>(P, P->r_gsum), task_count);
+  P->launches += 1;
+  if ((e = cudaGetLastError()) != cudaSuccess || GRID) return e;
+  const int64_t cells = P->nblk_interp * a.nacc;
+  ds_rows_kernel<<<unsigned((cells + 255) / 256), 256, 0, st>>>(
+      wsp<double>(P, P->r_gsum), a.ntask, a.nacc, a.nbw, a.b, P->nblk_interp,
+      wsp<double>(P, P->r_part));
   P->launches += 1;
   return cudaGetLastError();
 }
@@ -572,7 +591,6 @@ cudaError_t run_direct_interp(fkreg_plan_s* P, int b, int n_rhs_str, int n_probe
   a.nstr = n_rhs_str + n_probes;
   a.fields = P->ns + a.nstr * P->nt;
   a.ntask = (P->n + 31) / 32;
-  a.nblk_rows = P->nblk_interp;
   if (a.fields > kDirectMaxFields || a.nacc > kMaxAcc) return cudaErrorInvalidValue;
   return P->prec == FKREG_F32 ? run_ds<float, false>(P, a, 1, mhat_at_x, st)
                               : run_ds<double, false>(P, a, 1, mhat_at_x, st);

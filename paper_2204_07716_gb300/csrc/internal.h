@@ -174,7 +174,7 @@ struct fkreg_plan_s {
       r_binstart, r_nsub, r_substart, r_subbin, r_subfirst, r_hist, r_hist2, r_dtot, r_scan, r_str,
       r_fine, r_spec, r_gspec, r_gfield, r_t2spec, r_t2field, r_part, r_smax, r_fftwork,
       r_fftwork_g,
-      r_bV, r_bdx, r_bsc, r_gmask, r_gadj, r_gpart, r_gavec;
+      r_bV, r_bdx, r_bsc, r_gmask, r_gadj, r_gpart, r_gavec, r_gsum;
   bool backward = false;        // workspace reserved for fkreg_backward
   bool direct = false;          // compact kernel: direct sums instead of the NUFFT
   int f2bwd = 0;                // fields of the backward passes (one response + probes)

@@ -8,7 +8,9 @@
 //   rss_r      = sum_i (y_ri - mhat_r(x_i))^2                 (numerator of eq. 22)
 //   wSw_p      = sum_i w_pi (S w_p)_i,  ww_p = sum_i w_pi^2   (Sec. 2.1)
 //   tr_exact   = K_H(0) sum_i [S(x_i)^-1]_11                  (diagonal of S_h)
-// Block partials are summed in a fixed order, so results are deterministic.
+// Block partials are summed in a fixed order.  (Calls of the NUFFT path still differ in
+// rounding from run to run: the spreading adds its tiles with atomics, and the warps of
+// interp_direct.cu claim their groups.  The direct sums repeat bit for bit, direct.cu.)
 //
 // Fields are stored interleaved per fine-grid cell ([cell][rec], rec >= F2 an
 // odd number of 16-byte units), so a sample's fields of one cell are one
