@@ -13,9 +13,9 @@
 // each warp takes every fourth run of 32 samples, keeps those within reach of
 // the box, and when 32 are queued stages their strengths and walks them with
 // broadcast loads, every lane adding each to its own fields in registers.  The
-// warps' fields are added at the end.  Before, a warp held 32 samples and tested
-// every sample of the rows it staged (and the grid pass gave a warp to each
-// point and reduced every field over its lanes).  Four warps to 32 targets keep
+// warps' fields are added at the end.  (Before, a warp held 32 samples and tested
+// every sample of the rows it staged.)  Grids too coarse for patches have a warp
+// to each point (ds_patches).  Four warps to 32 targets keep
 // the chains short: with one warp to 32 targets and 128 to a block the same
 // instructions took four times as long, the schedulers idle nine cycles in ten
 // beside the blocks of dense regions.  Sums are taken in runs of 32
@@ -26,6 +26,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "device_common.cuh"
 #include "interp_common.cuh"
@@ -52,14 +53,12 @@ __host__ __device__ constexpr int ds_max_chunks() {
 }
 
 // Targets of a block of the grid pass: a patch of 4 x 8 (2-D) or 2 x 4 x 4 (3-D)
-// points, or 32 points in 1-D.
+// points.
 template <int D>
 __device__ __forceinline__ bool ds_grid_point(const GeoDev& g, int64_t task, int lane,
                                               int64_t (&m)[3]) {
   m[0] = m[1] = m[2] = 0;
-  if constexpr (D == 1) {
-    m[0] = task * 32 + lane;
-  } else if constexpr (D == 2) {
+  if constexpr (D == 2) {
     const int64_t nb1 = (g.M[1] + 7) / 8;
     m[0] = task / nb1 * 4 + (lane >> 3);
     m[1] = task % nb1 * 8 + (lane & 7);
@@ -79,7 +78,6 @@ __device__ __forceinline__ bool ds_grid_point(const GeoDev& g, int64_t task, int
 }
 
 inline int64_t ds_grid_tasks(const GeoDev& g, int d) {
-  if (d == 1) return (g.M[0] + 31) / 32;
   if (d == 2) return (g.M[0] + 3) / 4 * ((g.M[1] + 7) / 8);
   return (g.M[0] + 1) / 2 * ((g.M[1] + 3) / 4) * ((g.M[2] + 3) / 4);
 }
@@ -144,6 +142,7 @@ struct DsArgs {
   int str_pass;        // the strengths' pass (see kStrFlag)
   int64_t ntask;       // groups of 32 targets
   int64_t Mtot;        // grid: points
+  int slice;           // grid: field slice of the first bandwidth
 };
 
 // A target's fields.  add: one candidate of the walk, w its kernel value at this lane's target (0
@@ -458,7 +457,7 @@ direct_sums_kernel(GeoDev g, MonoTab mono, DsArgs a, const BwDev* __restrict__ b
 #pragma unroll
       for (int w = 1; w < kDsWarps; ++w) v += rows_f[(w * 32 + lane) * a.bstride + f];
       if constexpr (GRID) {
-        if (valid) field[(int64_t(blockIdx.y) * a.fields + f) * a.Mtot + idx] = v;
+        if (valid) field[(int64_t(a.slice + blockIdx.y) * a.fields + f) * a.Mtot + idx] = v;
       } else {
         rows_f[lane * a.bstride + f] = v;
       }
@@ -564,14 +563,49 @@ cudaError_t dispatch_ds(fkreg_plan_s* P, const DsArgs& a, int bw_count, void* mh
 template <typename T, bool GRID>
 cudaError_t run_ds(fkreg_plan_s* P, const DsArgs& a, int bw_count, void* mhat_at_x,
                    cudaStream_t st) {
-#define FK_DS(DD, OO) \
-  if (P->d == DD && P->order == OO) return dispatch_ds<T, DD, OO, GRID>(P, a, bw_count, mhat_at_x, st);
+#define FK_DS(DD, OO)                                                        \
+  if constexpr (!GRID || DD > 1) /* 1-D grids have a warp to each point */   \
+    if (P->d == DD && P->order == OO)                                        \
+      return dispatch_ds<T, DD, OO, GRID>(P, a, bw_count, mhat_at_x, st);
   FK_DS(1, 0) FK_DS(1, 1) FK_DS(1, 2) FK_DS(2, 0) FK_DS(2, 1) FK_DS(2, 2) FK_DS(3, 0) FK_DS(3, 1)
 #undef FK_DS
   return cudaErrorInvalidValue;
 }
 
 }  // namespace
+
+// Patches of 32 points, or a warp to each point (direct_points.cu)?  A patch walks
+// every sample within reach of its box, so its work per point grows by `reach`, the
+// box of support and patch against the support's; a warp per point adds only the
+// samples inside, in 32 lanes, and pays a fixed part of some hundred samples.  A
+// patch is also one block with a long chain: few of them leave SMs idle.  On a
+// GB300, over 660 random calls (1-D to 3-D, orders 0 to 2, 1 to 12 responses, 3000 to
+// 10^6 samples), us with patches and with points:
+//   FP32 2-D: 338^2 points, reach 1.2, 400 samples inside 220 / 610; 181^2, 1.6, 2200:
+//   397 / 473; 82 x 43, 2.8, 4700: 562 / 164; 16^2, 5.0, 530: 119 / 51;
+//   FP32 3-D: 53^3, 2.1, 67: 312 / 2488; 13^3, 3.3, 8500: 1655 / 343;
+//   FP64 2-D: 186^2, 2.5, 12: 190 / 524; 262^2, 3.4, 73: 1968 / 1417; 100^2, 3.5, 500:
+//   2610 / 614; FP64 3-D: 38^3, 2.3, 24: 762 / 3271; 18^3, 5.0, 3200: 21678 / 2518;
+//   1-D, where 32 points are a long box: 0.7 to 1.7 times in FP32 at reach below 2.1, 18
+//   times at 117; 1.5 to 72 times in FP64.
+// The rule loses 2 % on average against the better of the two, 1.6 times at most.
+static bool ds_patches(const fkreg_plan_s* P, int b) {
+  if (P->d == 1) return false;
+  const GeoDev& g = P->geo;
+  const BwDev& B = P->bw[b];
+  const int64_t patch[3] = {P->d == 2 ? 4 : 2, P->d == 2 ? 8 : 4, 4};
+  double reach = 1.0, inside = double(P->n) * (P->d == 2 ? M_PI : 4.0 / 3.0 * M_PI);
+  for (int j = 0; j < P->d; ++j) {
+    const double w = g.hi[j] - g.lo[j];
+    reach *= 1.0 + w * double(std::min(patch[j], g.M[j]) - 1) / double(g.M[j] - 1) / (2.0 * B.sigma[j]);
+    inside *= B.sigma[j] / w;
+  }
+  inside = std::min(inside, double(P->n));
+  const double idle = std::max(1.0, 4.0 * P->sm_count / double(ds_grid_tasks(g, P->d)));
+  return P->prec == FKREG_F32
+             ? 0.35 * reach * inside * idle < inside + 400.0
+             : reach * inside * idle < inside + 200.0;
+}
 
 cudaError_t run_direct_grid(fkreg_plan_s* P, int str_first, int nstr, int bw_first,
                             int bw_count, cudaStream_t st) {
@@ -585,8 +619,20 @@ cudaError_t run_direct_grid(fkreg_plan_s* P, int str_first, int nstr, int bw_fir
   a.Mtot = P->geo.M[0] * P->geo.M[1] * P->geo.M[2];
   if (a.fields > kDirectMaxFields) return cudaErrorInvalidValue;
   if (a.Mtot * bw_count == 0) return cudaSuccess;
-  return P->prec == FKREG_F32 ? run_ds<float, true>(P, a, bw_count, nullptr, st)
-                              : run_ds<double, true>(P, a, bw_count, nullptr, st);
+  for (int i = 0; i < bw_count;) {  // runs of bandwidths that take the same kernel
+    const bool patches = ds_patches(P, bw_first + i);
+    int k = i + 1;
+    while (k < bw_count && ds_patches(P, bw_first + k) == patches) ++k;
+    a.b = bw_first + i;
+    a.slice = i;
+    const cudaError_t e =
+        !patches ? run_direct_points(P, str_first, nstr, a.b, k - i, i, st)
+                 : (P->prec == FKREG_F32 ? run_ds<float, true>(P, a, k - i, nullptr, st)
+                                         : run_ds<double, true>(P, a, k - i, nullptr, st));
+    if (e != cudaSuccess) return e;
+    i = k;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t run_direct_interp(fkreg_plan_s* P, int b, int n_rhs_str, int n_probes,

@@ -307,6 +307,9 @@ cudaError_t run_interp(fkreg_plan_s* P, int b, int n_rhs_str, int n_probes, void
 // plus the s-fields, bandwidths [bw_first, bw_first + bw_count), into r_gfield
 cudaError_t run_direct_grid(fkreg_plan_s* P, int str_first, int nstr, int bw_first,
                             int bw_count, cudaStream_t s);
+// the same with a warp to each point, into the field slices from `slice` on
+cudaError_t run_direct_points(fkreg_plan_s* P, int str_first, int nstr, int bw_first, int bw_count,
+                              int slice, cudaStream_t s);
 cudaError_t run_direct_interp(fkreg_plan_s* P, int b, int n_rhs_str, int n_probes,
                               void* mhat_at_x, cudaStream_t s);
 cudaError_t run_finalize(fkreg_plan_s* P, int n_probes, const fkreg_outputs* out,
