@@ -18,9 +18,10 @@
 // to each point (ds_patches).  Four warps to 32 targets keep
 // the chains short: with one warp to 32 targets and 128 to a block the same
 // instructions took four times as long, the schedulers idle nine cycles in ten
-// beside the blocks of dense regions.  Sums are taken in runs of 32
+// beside the blocks of dense regions.  The grid pass sums in runs of 32
 // candidates that are then added to totals, so rounding grows with the root
-// of some tens, not of thousands.  A form on the tensor cores (split-TF32, 32
+// of some tens, not of thousands; at the samples a warp's quarter of the
+// candidates is one chain.  A form on the tensor cores (split-TF32, 32
 // targets x 8 candidates a step) was tried and left out: no faster, and the
 // truncating accumulators tripled the error against 64 bits.
 #include <cuda_runtime.h>

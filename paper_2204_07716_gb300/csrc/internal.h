@@ -26,6 +26,10 @@ constexpr int kSortTileKeys = 4096;  // keys per radix-sort tile (one block)
 // Up to 512 tiles' worth of samples the fused sort takes tiles of 1024 keys: a
 // scatter is bound by the serial work of one block (16 rounds of 4096 keys), so
 // a small problem is as slow as a large one unless its keys go to more blocks.
+// Estimates with tiles of 4096 and of 1024 keys, us: 1-D, 10,000 samples 135 / 115,
+// 520,000 samples 303 / 187; 2-D, 300,000 samples 196 / 170, 520,000 samples 224 / 212.
+// At 10^6 samples a block's fixed work (per-digit counts and scans) has won: the
+// 2-D step takes 677 us with 4096 keys and 692 with 1024.
 constexpr int kSmallTile = 1024;
 constexpr int64_t kSmallTileMaxN = 512 * kSmallTile;
 constexpr int64_t kFft1dMax = 4096;  // longest 1-D transform of fft1d.cu
@@ -94,16 +98,19 @@ inline int key_local_bits(int d, const int64_t* tile, const int64_t* nbins) {
 
 // Sub-problem size of a plan for up to max_n samples in nbins bins.  Where the
 // bins are fewer than two per SM they are split into about four sub-problems
-// per SM, so that a small problem fills the GPU (10,000 1-D samples in one
-// bin: 10 blocks of 1024 before, 40 of 256 now, a group of 32 for each warp).  More
-// bins than that give blocks enough by themselves, and every further split
-// pays for one more tile flush (16 strengths of a 24 x 24 tile against some
-// hundred samples: the GCV backward of 89,787 samples in 250 bins ran 10 % slower
-// with 160 than with 1024).  FP64 2-D blocks are long (the FP64 pipe) against
-// their flush: there the split also evens out the last wave, and so it does for
-// the 3-D FP32 spreading of width 7 (the only user of sub-problems in 3-D;
-// 300,001 samples in 336 bins, 1024 -> 512: the busiest SM had 1.4 times the
-// mean, a call took 932 -> 888 us).
+// per SM, so that a small problem fills the GPU.  With 1024 and with the rule, us:
+// 1-D FP64, 10,000 samples in one bin (256) 226 / 180; FP32 2-D, 30,000 samples in 63
+// bins (256), estimate with ten probes 227 / 189, GCV gradient 1134 / 1004; 90,000
+// samples (256) 189 / 177 and 1087 / 1059.  Every split pays for one more tile flush
+// (some strengths of a 24 x 24 tile against the sub-problem's samples), so no size is
+// below kSubMin, and where the bins hold many samples already the split no longer
+// gains: 520,000 samples in 63 bins (864) 292 / 300 and 1458 / 1492.  More bins than
+// two per SM give blocks enough by themselves.  FP64 2-D blocks are long (the FP64
+// pipe) against their flush: there the split also evens out the last wave (90 bins,
+// 30,000 samples 677 / 405; 520,000 samples 2660 / 2537), and so it does for the 3-D
+// FP32 spreading of width 7 (the only user of sub-problems in 3-D) with few strengths:
+// 300,001 samples in 336 bins, local linear (512) 932 / 888; with seventeen strengths
+// the flushes cost more than that gains: 200,000 samples in 294 bins (352) 1534 / 1626.
 inline uint32_t sub_problem_size(int d, int w, bool f64, int64_t nbins, int64_t max_n, int sm_count) {
   const int64_t sms = sm_count < 1 ? 1 : sm_count;
   if (d > 2 ? (f64 || w != 7) : (nbins >= 2 * sms && !f64)) return kSubMax;
