@@ -432,8 +432,8 @@ fkreg_status compute_geometry(const fkreg_opts* o, fkreg_geometry* g, std::strin
     // lands on the smaller, and the fields of a batch differ by the units of the box
     // to the second power (FP32, 1-D local linear, 5103 points, bandwidth 0.002: the
     // z^2 field 5e-2 off, the estimate 2e-3; 2-D, last axis 1029, box edge 1e-3: the
-    // estimate 4e-2).  Even lengths are transformed row by
-    // row, and so are all that the library transforms itself.
+    // estimate 4e-2).  Even lengths are transformed row by row, and so are all that the
+    // library transforms itself.
     const bool own = d == 1 && next_fast(L) <= kFft1dMax;
     L = j == d - 1 && !own ? next_fast_even(L) : next_fast(L);
     g->delta[j] = delta;
